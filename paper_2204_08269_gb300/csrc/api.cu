@@ -375,9 +375,11 @@ jtfs_status jtfs_plan_create(const jtfs_config* cfg, int64_t N, jtfs_plan** out)
   d.u1_len = p->u1_len; d.uh_len = p->uh_len; d.y_len = p->y_len;
   // psi-hat_alpha support end (xi + 8 sigma; both Morlet terms are below e^-32 past it) and the
   // row items of the batched second-order producer: G rows of one rate per CTA
-  long long off_yt = 0;
+  long long off_yt = 0, off_pw = 0;
   for (int a = 0; a < p->n2; ++a) {
     Rate2& A = p->rates2[a];
+    A.off_pw = (int)off_pw;
+    off_pw += A.L;
     A.k2e = (int)std::min<double>(d.K2max, std::floor((p->xi2[a] + kSupportSigmas * p->sg2[a]) * (double)N) + 1.0);
     A.kt = A.s ? (p->n1 - (A.lam_min & ~7) + 3) / 4 * 4 : 0;
     A.off_yt = off_yt;
@@ -422,6 +424,7 @@ jtfs_status jtfs_plan_create(const jtfs_config* cfg, int64_t N, jtfs_plan** out)
   const size_t o_psi2 = place(sizeof(float) * (size_t)p->n2 * d.K2max);
   const size_t o_phiT = place(sizeof(float) * N);
   const size_t o_phiTlo = place(sizeof(float) * N);
+  const size_t o_poolw = place(sizeof(float) * std::max<long long>(1, off_pw));
   // phi_T's spectrum on the bins it is built from (q <= 12 sigma_T N), FP64 then rounded
   const double sT = 0.1 / (double)p->cfg.T;
   d.phiT_kmax = std::min((int)std::ceil(12.0 * sT * N), (int)(N / 2));
@@ -449,6 +452,7 @@ jtfs_status jtfs_plan_create(const jtfs_config* cfg, int64_t N, jtfs_plan** out)
   d.psi2 = (const float*)(base + o_psi2);
   d.phiT = (const float*)(base + o_phiT);
   d.phiT_lo = (const float*)(base + o_phiTlo);
+  d.poolw = (const float*)(base + o_poolw);
   d.phiThat = (const float*)(base + o_phat);
   d.phiF = (const float*)(base + o_phiF);
   d.h = (const float2*)(base + o_h);

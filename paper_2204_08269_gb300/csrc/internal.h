@@ -37,6 +37,7 @@ struct Rate2 {
   int kt;       // lambda' columns of the transposed TF32 planes: from lam_min & ~7, padded to 4
   long long off_y;  // offset of Y_alpha (K x L complex) in a packed per-signal array
   long long off_yt; // offset of the transposed plane (L x kt) in a packed per-signal array
+  int off_pw;       // offset of the rate's L pooling weights in DevPlan.poolw
 };
 
 // Device-side constants of a plan (passed by value to kernels).
@@ -55,6 +56,8 @@ struct DevPlan {
   const float* psi2;      // [n2][K2max]
   const float* phiT;      // [N] time-domain lowpass phi_T[n]
   const float* phiT_lo;   // [N] phi_T[n] - phiT[n] (FP32), for the compensated S0 sums
+  const float* poolw;     // per kept rate its L weights s phi_T[(-m s) mod N]: the weight of sample
+                          // m in frame t is entry (m - t T / s) mod L of them
   const float* phiThat;   // [phiT_kmax + 1] its spectrum phi-hat(q / N), q = 0..phiT_kmax (the
                           // bins phi_T is built from; beyond them phi-hat < e^-72)
   int phiT_kmax;

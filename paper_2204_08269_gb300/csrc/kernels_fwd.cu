@@ -279,38 +279,118 @@ __global__ void k_transpose_yt(DevPlan P, int a, const float* __restrict__ y,
   }
 }
 
+// Time pooling of one real row of L samples at a stride of L / (tau n_t) (tau = T / s samples per
+// frame): out(t) = sum_m w[(m - t tau) mod L] a[m] with the rate's weights w (DevPlan.poolw), for
+// the FB frames from t0, summed over the calling warp's share of the samples.  With m = q tau +
+// rho the FB frames' weights of consecutive q are a sliding window over w: each step loads one
+// weight and one sample for FB products (a weight per product would leave the kernel bound by
+// its loads).  Lanes take consecutive rho, so a warp's loads are contiguous; a row with fewer than
+// 32 samples per frame takes lanes over m and loads every weight.  Warp `seg` of `segs` takes
+// every segs-th block of 32 rho.  The lanes' partials are summed by a butterfly that halves the
+// frames per lane: on return lane l holds frame t0 + (l >> (5 - log2 FB)).
+template <int FB>
+__device__ __forceinline__ float pool_row_frames(const float2* sm, int row0, int logL, int tau,
+                                                 int nt, int t0, const float* __restrict__ w,
+                                                 int seg, int segs, int lane) {
+  const int L = 1 << logL;
+  float acc[FB];
+#pragma unroll
+  for (int j = 0; j < FB; ++j) acc[j] = 0.f;
+  if (tau >= 32) {
+    for (int rho = 32 * seg + lane; rho < tau; rho += 32 * segs) {
+      // slot (q - j) mod FB holds the weight of frame t0 + j at step q
+      float win[FB];
+#pragma unroll
+      for (int j = 1; j < FB; ++j) win[FB - j] = __ldg(&w[((nt - t0 - j) & (nt - 1)) * tau + rho]);
+      for (int q0 = 0; q0 < nt; q0 += FB) {
+#pragma unroll
+        for (int e = 0; e < FB; ++e) {
+          const int q = q0 + e;
+          win[e] = __ldg(&w[((q - t0) & (nt - 1)) * tau + rho]);
+          const float v = sm[fft_pos(row0 + q * tau + rho, logL)].x;
+#pragma unroll
+          for (int j = 0; j < FB; ++j) acc[j] = fmaf(win[(e - j + FB) & (FB - 1)], v, acc[j]);
+        }
+      }
+    }
+  } else {
+    for (int m = 32 * seg + lane; m < L; m += 32 * segs) {
+      const float v = sm[fft_pos(row0 + m, logL)].x;
+#pragma unroll
+      for (int j = 0; j < FB; ++j) acc[j] = fmaf(__ldg(&w[(m - (t0 + j) * tau) & (L - 1)]), v, acc[j]);
+    }
+  }
+  int o = 16;
+#pragma unroll
+  for (int h = FB / 2; h > 0; h >>= 1, o >>= 1) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int j = 0; j < h; ++j) {
+      const float give = up ? acc[j] : acc[j + h], keep = up ? acc[j + h] : acc[j];
+      acc[j] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+    }
+  }
+  for (; o > 0; o >>= 1) acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], o);
+  return acc[0];
+}
+
 // Time scattering (Scattering1D, the baseline of Sec. 4.4): the second order without the
 // log-frequency stage, S2t[alpha][lambda'][t] = sum_m s_alpha phi_T[(t T - m s_alpha) mod N]
 // |Y_alpha[lambda'][m]|.  One CTA per G rows of one rate: the rows are folded and inverse
 // transformed in shared memory as for the Y producer, their moduli replace them there, and
-// each warp reduces one (row, frame) output at a time; Y never leaves the chip.
-__global__ void __launch_bounds__(kRowBound)
+// the warps pool FB frames of a row at a time (pool_row_frames); Y never leaves the chip.  With
+// fewer rows than warps, `segs` warps share a row and their partials are added in order.
+// B = 32, N = 2^16, 167 rows, 32 frames: 5.20 -> 0.66 ms.  One warp per (row, frame) that gathered
+// phi_T at the rate's stride spent it on weight loads (32 sectors per warp and product); now the
+// fold and the FFT passes bound it, as they do the Y producer.
+constexpr int kPoolPartNt = 64;   // frames up to which warps share a row
+
+template <int FB>
+__global__ void __launch_bounds__(kRowThreads)
 k_scat1d_rows(DevPlan P, const int4* __restrict__ items, const float2* __restrict__ uh,
               float* __restrict__ s2t) {
   extern __shared__ float2 sm[];
-  __shared__ int s_off[kMaxRowsPerItem], s_kend[kMaxRowsPerItem];
-  __shared__ float s_inv[kMaxRowsPerItem];
+  // the row tables, then (once the moduli are taken) the partials of shared rows: one array, so
+  // that three 256-thread blocks still fit an SM
+  __shared__ int s_tab[3 * kMaxRowsPerItem];
+  int *s_off = s_tab, *s_kend = s_tab + kMaxRowsPerItem;
+  float* s_inv = reinterpret_cast<float*>(s_tab + 2 * kMaxRowsPerItem);
+  float* part = reinterpret_cast<float*>(s_tab);
+  static_assert((kRowThreads / 32) * kPoolPartNt <= 3 * kMaxRowsPerItem, "partials");
   const int4 it = items[blockIdx.x];
   const int a = it.x, lam0 = it.y, G = it.z, b = blockIdx.y;
   const Rate2 A = P.rates2[a];
-  const int L = A.L, logL = A.logL, nt = P.n_t;
+  const int L = A.L, logL = A.logL, nt = P.n_t, tau = P.T / A.s;
   second_order_rows_ifft(P, A, a, lam0, G, uh + (size_t)b * P.uh_len, sm, s_off, s_kend, s_inv);
   __syncthreads();
   for (int idx = threadIdx.x; idx < G * L; idx += blockDim.x) {
-    const float2 v = sm[fft_pos(idx, logL)];
-    sm[fft_pos(idx, logL)].x = sqrtf(v.x * v.x + v.y * v.y) * s_inv[idx >> logL];
+    const int at = fft_pos(idx, logL);
+    const float2 v = sm[at];
+    sm[at].x = sqrtf(v.x * v.x + v.y * v.y) * s_inv[idx >> logL];
   }
   __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  for (int o = warp; o < G * nt; o += nw) {
-    const int r = o / nt, t = o - r * nt;
-    float acc = 0.f;
-    for (int m = lane; m < L; m += 32)
-      acc = fmaf(__ldg(&P.phiT[((long long)t * P.T - (long long)m * A.s) & (P.N - 1)]),
-                 sm[fft_pos((r << logL) + m, logL)].x, acc);
-    for (int q = 16; q > 0; q >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, q);
-    if (lane == 0)
-      s2t[(((size_t)b * P.n2 + a) * P.n1 + lam0 + r) * nt + t] = acc * (float)A.s;
+  int segs = 1;
+  while (nt <= kPoolPartNt && 2 * segs * G <= nw && 32 * 2 * segs <= tau) segs <<= 1;
+  float* out = s2t + (((size_t)b * P.n2 + a) * P.n1 + lam0) * nt;
+  const float* w = P.poolw + A.off_pw;
+  constexpr int LPF = 32 / FB;    // lanes holding one frame's sum
+  for (int o = warp; o < G * segs; o += nw) {
+    const int r = o % G, seg = o / G;
+    for (int t0 = 0; t0 < nt; t0 += FB) {
+      const float v = pool_row_frames<FB>(sm, r << logL, logL, tau, nt, t0, w, seg, segs, lane);
+      if (lane % LPF == 0) {
+        const int i = r * nt + t0 + lane / LPF;
+        if (segs == 1) out[i] = v; else part[seg * G * nt + i] = v;
+      }
+    }
+  }
+  if (segs == 1) return;
+  __syncthreads();
+  for (int i = threadIdx.x; i < G * nt; i += blockDim.x) {
+    float v = 0.f;
+    for (int q = 0; q < segs; ++q) v += part[q * G * nt + i];
+    out[i] = v;
   }
 }
 
@@ -337,7 +417,9 @@ jtfs_status set_attrs(const jtfs_plan* p) {
   if ((st = cuda_check(cudaFuncSetAttribute(k_second_order_rows<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, rows_smem), "attr")) != JTFS_OK) return st;
   if ((st = cuda_check(cudaFuncSetAttribute(k_second_order_rows<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, rows_smem), "attr")) != JTFS_OK) return st;
   if ((st = cuda_check(cudaFuncSetAttribute(k_joint_fwd_simt, cudaFuncAttributeMaxDynamicSharedMemorySize, big), "attr")) != JTFS_OK) return st;
-  if ((st = cuda_check(cudaFuncSetAttribute(k_scat1d_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, rows_smem), "attr")) != JTFS_OK) return st;
+  for (const void* f : {(const void*)k_scat1d_rows<1>, (const void*)k_scat1d_rows<2>,
+                        (const void*)k_scat1d_rows<4>, (const void*)k_scat1d_rows<8>})
+    if ((st = cuda_check(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, rows_smem), "attr")) != JTFS_OK) return st;
   g_attrs_set[p->device] = true;
   return JTFS_OK;
 }
@@ -457,8 +539,12 @@ jtfs_status launch_scat1d_forward(const jtfs_plan* p, const float* x, int B, flo
     return rc;
   if (!p->rowitems.empty()) {
     StageScope sc(p, kStSecondOrder, st, 1);
-    k_scat1d_rows<<<dim3((unsigned)(p->rowitems.size() / 4), B), p->row_threads,
-                    (size_t)p->rows_cap * 17 / 2, st>>>(
+    // eight frames per step of the pooling, or all of them
+    auto* kernel = p->n_t >= 8 ? k_scat1d_rows<8>
+                   : p->n_t == 4 ? k_scat1d_rows<4>
+                   : p->n_t == 2 ? k_scat1d_rows<2> : k_scat1d_rows<1>;
+    kernel<<<dim3((unsigned)(p->rowitems.size() / 4), B), p->row_threads,
+             (size_t)p->rows_cap * 17 / 2, st>>>(
         d, reinterpret_cast<const int4*>(p->d_rowitems), w.uh, s2t);
   }
   return cuda_check(cudaGetLastError(), "time scattering forward");

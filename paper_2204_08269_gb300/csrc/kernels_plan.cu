@@ -92,6 +92,14 @@ __global__ void k_fill_phiT(int N, int kmax, double sphi, float* out, float* out
   }
 }
 
+// Time-pooling weights of every kept rate, s phi_T[(-m s) mod N] for m < L (the other frames'
+// weights are circular shifts of them by T / s samples).
+__global__ void k_fill_poolw(DevPlan P, float* out) {
+  const Rate2 A = P.rates2[blockIdx.y];
+  for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < A.L; m += gridDim.x * blockDim.x)
+    out[A.off_pw + m] = P.phiT[(P.N - m * A.s) & (P.N - 1)] * (float)A.s;
+}
+
 // Log-frequency filters on the N_fr grid: h_c[m] = (1/N_fr) sum_j H_c(w_j) exp(2 pi i j m / N_fr),
 // H_c = c_fr psi(w) (theta = +1, c < n_fr), c_fr psi(-w) (theta = -1), phi_F(w) (c = 2 n_fr).
 __global__ void k_fill_fr(int Nfr, int nfr, const double* __restrict__ xi,
@@ -201,6 +209,7 @@ jtfs_status build_tables(jtfs_plan* p) {
     kmax = std::min(kmax, N / 2);
     k_fill_phiT<<<(N + 255) / 256, 256>>>(N, kmax, sT, const_cast<float*>(d.phiT),
                                           const_cast<float*>(d.phiT_lo));
+    k_fill_poolw<<<dim3(16, p->n2), 256>>>(d, const_cast<float*>(d.poolw));
   }
   if ((st = cuda_check(cudaDeviceSynchronize(), "k_fill_phiT")) != JTFS_OK) goto done;
   if ((st = upload(p->xi_fr, p->sg_fr)) != JTFS_OK) goto done;
