@@ -102,7 +102,6 @@ jtfs_status validate_cfg(const jtfs_config* c, int64_t N) {
 
 bool joint_simt_supported(const jtfs_plan* p);
 size_t joint_fwd_smem(const jtfs_plan* p);
-size_t joint_bwd_smem(const jtfs_plan* p);
 
 static cudaEvent_t take_event(Profiler& pr) {
   if (!pr.pool.empty()) {

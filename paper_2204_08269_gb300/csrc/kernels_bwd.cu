@@ -36,128 +36,208 @@ k_uh_from_u1(DevPlan P, const float* __restrict__ u1, float2* __restrict__ uh) {
 }
 
 // ---------------------------------------------------------------------------------------
-constexpr int kJT = 256;
-constexpr int kNC = 32;
-constexpr int kRPT = 8;
+// Joint backward on CUDA cores (plain FP32 plans, and the rates past the tensor-core form's
+// lambda' range).  One CTA per (alpha, NC-column chunk, signal); it walks the spin pairs and then
+// the phi_F channel, whose filters W = Wr + i Wi serve both spins (the spin-down filter is the
+// conjugate of the spin-up one), so four real products per (row, lambda', column) give both Z:
+//   [P1 | P3] = Wr [Yr | Yi], [P4 | P2] = Wi [Yr | Yi],
+//   Z_up = (P1 - P2) + i (P3 + P4), Z_down = (P1 + P2) + i (P3 - P4),
+// and with S = gZ_up + gZ_down, T = (Im gZ_up - Im gZ_down) + i (Re gZ_down - Re gZ_up) the adjoint
+// is gY += Wr^T S + Wi^T T (phi_F: Wi = 0, T unused).  Both products are bound by their FMAs: a
+// thread owns 8 consecutive rows x 4 columns, W is Toeplitz, so consecutive k shift an 8-entry
+// window of h by one and a step loads one h and four columns for 64 packed FMAs.  The gY
+// accumulators rest in shared memory while the Z product holds the registers.
+// B = 16, N = 2^17, the five lowest rates (167 lambda' rows): 6.00 -> 1.44 ms; the
+// earlier form took every spin by itself and loaded one h per four complex products.
+constexpr int kJR = 8;        // rows (or lambda') of a thread
+constexpr int kJC = 4;        // columns of a thread
+constexpr int kJT = 256;      // most threads: 256 / kJR row groups x 32 / kJC column groups
 
+struct JointBwdLayout {       // float offsets in shared memory
+  int rows, threads, y, st, gacc, h, g1, wt, total;
+};
+
+__host__ __device__ inline JointBwdLayout joint_bwd_layout(int n1, int nt, int nc) {
+  JointBwdLayout s;
+  s.rows = (n1 + kJR - 1) / kJR * kJR;
+  s.threads = (s.rows / kJR * (nc / kJC) + 31) / 32 * 32;
+  s.st = 0;                                   // [rows][nc] (S, T)
+  s.y = s.st + s.rows * nc * 4;               // [rows][nc] Y
+  s.gacc = s.y + s.rows * nc * 2;             // [2 kJR kJC][threads]
+  s.wt = s.gacc + 2 * kJR * kJC * s.threads;  // [nt][nc]
+  s.h = s.wt + nt * nc;                       // h[d], -rows <= d < rows
+  s.g1 = s.h + 4 * s.rows;                    // [2 spins][n1][nt]
+  s.total = s.g1 + 2 * n1 * nt;
+  return s;
+}
+
+template <int NC>
 __global__ void __launch_bounds__(kJT)
 k_joint_bwd_simt(DevPlan P, const int2* __restrict__ items, const float2* __restrict__ y,
                  const float* __restrict__ gs2, float2* __restrict__ gy) {
   extern __shared__ float4 smraw[];
+  float* smf = reinterpret_cast<float*>(smraw);
   const int2 it = items[blockIdx.x];
-  const int a = it.x, n0 = it.y, b = blockIdx.y;
+  const int a = it.x, n0 = it.y + (int)blockIdx.z * NC, b = blockIdx.y;
   const Rate2 A = P.rates2[a];
+  if (n0 >= A.L) return;
   const int n1 = P.n1, nt = P.n_t, K = A.K, l0 = A.lam_min, nfm = P.N_fr - 1;
-  float2* sh = reinterpret_cast<float2*>(smraw);        // [N_fr]
-  float2* yt = sh + P.N_fr;                              // [K][kNC]
-  float2* gz = yt + (size_t)n1 * kNC;                    // [n1][kNC]
-  float* g1 = reinterpret_cast<float*>(gz + (size_t)n1 * kNC);  // [n1][n_t]
-  float* wt = g1 + (size_t)n1 * nt;                      // [n_t][kNC]
+  const JointBwdLayout lay = joint_bwd_layout(n1, nt, NC);
+  const int Kp = (K + kJR - 1) / kJR * kJR, Rp = lay.rows;
+  float4* st = reinterpret_cast<float4*>(smf + lay.st);
+  float2* yt = reinterpret_cast<float2*>(smf + lay.y);
+  float* gacc = smf + lay.gacc;
+  float* wt = smf + lay.wt;
+  float2* sh = reinterpret_cast<float2*>(smf + lay.h) + Rp;   // sh[d], -Rp <= d < Rp
+  float* g1 = smf + lay.g1;
+  const int tid = threadIdx.x, nthr = blockDim.x;
   const float2* ya = y + (size_t)b * P.y_len + A.off_y;
-  for (int i = threadIdx.x; i < K * kNC; i += blockDim.x) {
-    const int k = i / kNC, col = i % kNC;
-    yt[i] = (n0 + col < A.L) ? ya[(size_t)k * A.L + n0 + col] : make_float2(0.f, 0.f);
+  for (int i = tid; i < Kp * NC; i += nthr) {
+    const int k = i / NC, col = i % NC;
+    yt[i] = (k < K && n0 + col < A.L) ? ya[(size_t)k * A.L + n0 + col] : make_float2(0.f, 0.f);
   }
-  for (int i = threadIdx.x; i < nt * kNC; i += blockDim.x) {
-    const int t = i / kNC, col = i % kNC;
-    const int n = n0 + col;
+  for (int i = tid; i < nt * NC; i += nthr) {
+    const int t = i / NC, n = n0 + i % NC;
     wt[i] = (n < A.L) ? __ldg(&P.phiT[(t * P.T - n * A.s) & (P.N - 1)]) * (float)A.s : 0.f;
   }
-  const int ty = threadIdx.x >> 3, tx = threadIdx.x & 7;
-  float2 gacc[kRPT][4];
-#pragma unroll
-  for (int i = 0; i < kRPT; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) gacc[i][j] = make_float2(0.f, 0.f);
+  for (int i = 0; i < 2 * kJR * kJC; ++i) gacc[i * nthr + tid] = 0.f;
+  // columns col0 + CS j: neighbouring lanes read neighbouring columns
+  constexpr int CS = NC / kJC;
+  const int col0 = tid % CS, r0 = tid / CS * kJR;
+  const bool has_rows = r0 < Rp, has_k = r0 < Kp;
 
-  for (int c = 0; c < P.C; ++c) {
+  for (int p = 0; p <= P.n_fr; ++p) {
+    const bool pair = p < P.n_fr;               // a spin pair, or the phi_F channel
+    const int c = pair ? p : 2 * P.n_fr;
     __syncthreads();
-    for (int i = threadIdx.x; i < P.N_fr; i += blockDim.x) sh[i] = P.h[(size_t)c * P.N_fr + i];
-    const float* g = gs2 + (size_t)b * P.s2_stride + ((size_t)a * P.C + c) * P.n_lo * nt;
-    for (int i = threadIdx.x; i < n1 * nt; i += blockDim.x) {
+    for (int i = tid; i < 2 * Rp; i += nthr)
+      sh[i - Rp] = P.h[(size_t)c * P.N_fr + ((i - Rp) & nfm)];
+    for (int i = tid; i < (pair ? 2 : 1) * n1 * nt; i += nthr) {
+      const int d = i >= n1 * nt ? 1 : 0, j = i - d * n1 * nt;
+      const float* g = gs2 + (size_t)b * P.s2_stride +
+                       ((size_t)a * P.C + c + d * P.n_fr) * P.n_lo * nt;
+      float v;
       if (P.average_fr) {
-        const int r = i / nt, t = i % nt;
-        float s = 0.f;
+        const int r = j / nt, t = j - r * nt;
+        v = 0.f;
         for (int lo = 0; lo < P.n_lo; ++lo)
-          s += __ldg(&P.phiF[(lo * P.s_F - r) & nfm]) * g[lo * nt + t];
-        g1[i] = s;
+          v += __ldg(&P.phiF[(lo * P.s_F - r) & nfm]) * __ldg(&g[lo * nt + t]);
       } else {
-        g1[i] = g[i];
+        v = g[j];
       }
+      g1[i] = v;
     }
     __syncthreads();
-    // Z = W_c Y for the thread's (row, column) outputs
-    float2 acc[kRPT][4];
+    // the products: pw = Wr Y, pi = Wi Y of rows r0 + i, columns col0 + CS j
+    float2 pw[kJR][kJC], pi[kJR][kJC];
 #pragma unroll
-    for (int i = 0; i < kRPT; ++i)
+    for (int i = 0; i < kJR; ++i)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) acc[i][j] = make_float2(0.f, 0.f);
-    for (int k = 0; k < K; ++k) {
-      const float4 y01 = reinterpret_cast<const float4*>(yt + k * kNC)[tx * 2];
-      const float4 y23 = reinterpret_cast<const float4*>(yt + k * kNC)[tx * 2 + 1];
-      const float2 yv[4] = {make_float2(y01.x, y01.y), make_float2(y01.z, y01.w),
-                            make_float2(y23.x, y23.y), make_float2(y23.z, y23.w)};
-      const int kk = k + l0;
+      for (int j = 0; j < kJC; ++j) pw[i][j] = pi[i][j] = make_float2(0.f, 0.f);
+    if (has_rows) {
+      // row i's filter entry at step k is h[r0 + i - k - l0], in slot (i - k) mod 8
+      float2 win[kJR];
 #pragma unroll
-      for (int i = 0; i < kRPT; ++i) {
-        const int r = ty + 32 * i;
+      for (int i = 1; i < kJR; ++i) win[i] = sh[r0 + i - l0];
+      for (int k0 = 0; k0 < Kp; k0 += kJR) {
+#pragma unroll
+        for (int e = 0; e < kJR; ++e) {
+          const int k = k0 + e;
+          win[(kJR - e) & (kJR - 1)] = sh[max(r0 - k - l0, -Rp)];
+          float2 yv[kJC];
+#pragma unroll
+          for (int j = 0; j < kJC; ++j) yv[j] = yt[k * NC + col0 + CS * j];
+#pragma unroll
+          for (int i = 0; i < kJR; ++i) {
+            const float2 w = win[(i - e + kJR) & (kJR - 1)];
+#pragma unroll
+            for (int j = 0; j < kJC; ++j) {
+              pw[i][j] = __ffma2_rn(make_float2(w.x, w.x), yv[j], pw[i][j]);
+              pi[i][j] = __ffma2_rn(make_float2(w.y, w.y), yv[j], pi[i][j]);
+            }
+          }
+        }
+      }
+      // g|Z| of both spins from the pooling adjoint, gZ = g|Z| Z / |Z|, then S and T
+#pragma unroll
+      for (int i = 0; i < kJR; ++i) {
+        const int r = r0 + i;
+        float gu[kJC] = {0.f, 0.f, 0.f, 0.f}, gd[kJC] = {0.f, 0.f, 0.f, 0.f};
         if (r < n1) {
-          const float2 hv = sh[(r - kk) & nfm];
+          const float *gur = g1 + r * nt, *gdr = gur + n1 * nt;
+          for (int t = 0; t < nt; ++t) {
+            const float u = gur[t], d = pair ? gdr[t] : 0.f;
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            acc[i][j].x += hv.x * yv[j].x - hv.y * yv[j].y;
-            acc[i][j].y += hv.x * yv[j].y + hv.y * yv[j].x;
+            for (int j = 0; j < kJC; ++j) {
+              const float wv = wt[t * NC + col0 + CS * j];
+              gu[j] = fmaf(u, wv, gu[j]);
+              gd[j] = fmaf(d, wv, gd[j]);
+            }
           }
         }
-      }
-    }
-    // g|Z| = sum_t g1[r][t] w[t][col];  gZ = g|Z| Z / |Z|
 #pragma unroll
-    for (int i = 0; i < kRPT; ++i) {
-      const int r = ty + 32 * i;
-      if (r < n1) {
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const int col = tx * 4 + j;
-          float ga = 0.f;
-          for (int t = 0; t < nt; ++t) ga += g1[r * nt + t] * wt[t * kNC + col];
-          const float2 z = acc[i][j];
-          const float m = sqrtf(z.x * z.x + z.y * z.y);
-          const float f = (m > 0.f) ? ga / m : 0.f;
-          gz[r * kNC + col] = make_float2(z.x * f, z.y * f);
+        for (int j = 0; j < kJC; ++j) {
+          const float2 w = pw[i][j], q = pi[i][j];
+          const float2 zu = make_float2(w.x - q.y, w.y + q.x), zd = make_float2(w.x + q.y, w.y - q.x);
+          const float mu = sqrtf(zu.x * zu.x + zu.y * zu.y), md = sqrtf(zd.x * zd.x + zd.y * zd.y);
+          const float fu = mu > 0.f ? gu[j] / mu : 0.f, fd = md > 0.f ? gd[j] / md : 0.f;
+          const float2 zgu = make_float2(zu.x * fu, zu.y * fu), zgd = make_float2(zd.x * fd, zd.y * fd);
+          st[r * NC + col0 + CS * j] =
+              pair ? make_float4(zgu.x + zgd.x, zgu.y + zgd.y, zgu.y - zgd.y, zgd.x - zgu.x)
+                   : make_float4(zgu.x, zgu.y, 0.f, 0.f);
         }
       }
     }
     __syncthreads();
-    // gY[k][col] += sum_r conj(h_c[(r - k) mod N_fr]) gZ[r][col]
-    for (int r = 0; r < n1; ++r) {
-      const float4 g01 = reinterpret_cast<const float4*>(gz + r * kNC)[tx * 2];
-      const float4 g23 = reinterpret_cast<const float4*>(gz + r * kNC)[tx * 2 + 1];
-      const float2 gv[4] = {make_float2(g01.x, g01.y), make_float2(g01.z, g01.w),
-                            make_float2(g23.x, g23.y), make_float2(g23.z, g23.w)};
+    if (has_k) {
+      // gY[k][col] += sum_r Wr[r][k] S[r][col] + Wi[r][k] T[r][col], k = r0 + i: the filter entry
+      // h[r - k - l0] is in slot (r - i) mod 8
+      float2 acc[kJR][kJC];
 #pragma unroll
-      for (int i = 0; i < kRPT; ++i) {
-        const int k = ty + 32 * i;
-        if (k < K) {
-          const float2 hv = sh[(r - k - l0) & nfm];
+      for (int i = 0; i < kJR; ++i)
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            gacc[i][j].x += hv.x * gv[j].x + hv.y * gv[j].y;
-            gacc[i][j].y += hv.x * gv[j].y - hv.y * gv[j].x;
+        for (int j = 0; j < kJC; ++j)
+          acc[i][j] = make_float2(gacc[2 * (i * kJC + j) * nthr + tid],
+                                  gacc[(2 * (i * kJC + j) + 1) * nthr + tid]);
+      float2 win[kJR];
+#pragma unroll
+      for (int i = 1; i < kJR; ++i) win[kJR - i] = sh[max(-(r0 + i) - l0, -Rp)];
+      for (int rr = 0; rr < Rp; rr += kJR) {
+#pragma unroll
+        for (int e = 0; e < kJR; ++e) {
+          const int r = rr + e;
+          win[e] = sh[max(r - r0 - l0, -Rp)];
+#pragma unroll
+          for (int j = 0; j < kJC; ++j) {
+            const float4 v = st[r * NC + col0 + CS * j];
+#pragma unroll
+            for (int i = 0; i < kJR; ++i) {
+              const float2 w = win[(e - i + kJR) & (kJR - 1)];
+              acc[i][j] = __ffma2_rn(make_float2(w.x, w.x), make_float2(v.x, v.y), acc[i][j]);
+              acc[i][j] = __ffma2_rn(make_float2(w.y, w.y), make_float2(v.z, v.w), acc[i][j]);
+            }
           }
         }
       }
+#pragma unroll
+      for (int i = 0; i < kJR; ++i)
+#pragma unroll
+        for (int j = 0; j < kJC; ++j) {
+          gacc[2 * (i * kJC + j) * nthr + tid] = acc[i][j].x;
+          gacc[(2 * (i * kJC + j) + 1) * nthr + tid] = acc[i][j].y;
+        }
     }
   }
   float2* go = gy + (size_t)b * P.y_len + A.off_y;
+  if (has_k) {
 #pragma unroll
-  for (int i = 0; i < kRPT; ++i) {
-    const int k = ty + 32 * i;
-    if (k < K)
+    for (int i = 0; i < kJR; ++i)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int col = tx * 4 + j;
-        if (n0 + col < A.L) go[(size_t)k * A.L + n0 + col] = gacc[i][j];
+      for (int j = 0; j < kJC; ++j) {
+        const int k = r0 + i, n = n0 + col0 + CS * j;
+        if (k < K && n < A.L)
+          go[(size_t)k * A.L + n] = make_float2(gacc[2 * (i * kJC + j) * nthr + tid],
+                                                gacc[(2 * (i * kJC + j) + 1) * nthr + tid]);
       }
   }
 }
@@ -481,7 +561,8 @@ jtfs_status set_attrs(const jtfs_plan* p) {
   std::lock_guard<std::mutex> lk(g_attrs_mu);
   if (g_attrs_set[p->device]) return JTFS_OK;
   const int big = 227 * 1024;
-  const void* fns[] = {(const void*)k_uh_from_u1, (const void*)k_joint_bwd_simt,
+  const void* fns[] = {(const void*)k_uh_from_u1, (const void*)k_joint_bwd_simt<32>,
+                       (const void*)k_joint_bwd_simt<16>,
                        (const void*)k_second_order_bwd, (const void*)k_stage1_bwd,
                        (const void*)k_gx, (const void*)k_xfft_sub};
   for (const void* f : fns) {
@@ -505,9 +586,16 @@ jtfs_status set_attrs(const jtfs_plan* p) {
 
 }  // namespace
 
-size_t joint_bwd_smem(const jtfs_plan* p) {
-  return (size_t)p->N_fr * 8 + 2 * (size_t)p->n1 * kNC * 8 + (size_t)p->n1 * p->n_t * 4 +
-         (size_t)p->n_t * kNC * 4;
+// The CUDA-core joint backward over 32-column items: 32 columns at a time where the shared memory
+// holds them (every configuration but those with many rows and frames), else 16.
+static void launch_joint_bwd_simt(const jtfs_plan* p, int n_items, const int* items, int B,
+                                  const float2* y, const float* gs2, float2* gy, cudaStream_t st) {
+  const JointBwdLayout w = joint_bwd_layout(p->n1, p->n_t, 32);
+  const bool wide = (size_t)w.total * 4 <= 227 * 1024;
+  const JointBwdLayout l = wide ? w : joint_bwd_layout(p->n1, p->n_t, 16);
+  auto* kernel = wide ? k_joint_bwd_simt<32> : k_joint_bwd_simt<16>;
+  kernel<<<dim3((unsigned)n_items, B, wide ? 1 : 2), l.threads, (size_t)l.total * 4, st>>>(
+      p->dp, reinterpret_cast<const int2*>(items), y, gs2, gy);
 }
 
 bool backward_reuses_forward(const jtfs_plan* p) {
@@ -555,9 +643,8 @@ jtfs_status launch_backward(const jtfs_plan* p, const float* x, const float* u1,
                               p->row_threads, (size_t)p->tcb_fb_cap * 17 / 2, st>>>(
           d, reinterpret_cast<const int4*>(p->d_tcb_fb_rowitems), w.uh, w.y, nullptr, nullptr,
           B);
-      k_joint_bwd_simt<<<dim3((unsigned)(p->tcb_fb_items.size() / 2), B), kJT,
-                         joint_bwd_smem(p), st>>>(
-          d, reinterpret_cast<const int2*>(p->d_tcb_fb_items), w.y, gs2, w.gy);
+      launch_joint_bwd_simt(p, (int)(p->tcb_fb_items.size() / 2), p->d_tcb_fb_items, B, w.y, gs2,
+                            w.gy, st);
       p->prof.launches += 2;
     }
   } else if (gs2 && n_items > 0) {
@@ -568,8 +655,7 @@ jtfs_status launch_backward(const jtfs_plan* p, const float* x, const float* u1,
           d, reinterpret_cast<const int4*>(p->d_rowitems), w.uh, w.y, nullptr, nullptr, B);
     }
     StageScope sc(p, kStJointBwd, st, 1);
-    k_joint_bwd_simt<<<dim3((unsigned)n_items, B), kJT, joint_bwd_smem(p), st>>>(
-        d, reinterpret_cast<const int2*>(p->d_items), w.y, gs2, w.gy);
+    launch_joint_bwd_simt(p, (int)n_items, p->d_items, B, w.y, gs2, w.gy, st);
   } else if (p->y_len > 0) {
     cudaMemsetAsync(w.gy, 0, (size_t)B * p->y_len * sizeof(float2), st);
   }
