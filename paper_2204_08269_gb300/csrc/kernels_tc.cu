@@ -165,7 +165,7 @@ k_joint_fwd_tc(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
-    if (lane == 0) {
+    if (elect_one()) {
       int stage = 0, ws = 0;
       uint32_t phase = 0, wph = 0, aph = 0;
       // stages / weight buffers with a load in flight, and the parity each one completes
@@ -232,7 +232,7 @@ k_joint_fwd_tc(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
+    if (elect_one()) {
       const uint32_t id_pos = instr_desc(kBM, BN, 1, 1, 0, 1, 0);
       const uint32_t id_neg = instr_desc(kBM, BN, 1, 1, 0, 1, 1);
       const uint32_t id_pool = instr_desc(kBM, NT, 1, 1, 0, 0, 0);
@@ -918,7 +918,7 @@ k_joint_fwd_tp(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
-    if (lane == 0) {
+    if (elect_one()) {
       int stage = 0, ws = 0;
       uint32_t phase = 0, wph = 0, aph = 0;
       uint32_t armed = 0, armed_par = 0, armed_w = 0, armed_w_par = 0;
@@ -978,7 +978,7 @@ k_joint_fwd_tp(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ product issuer
-    if (lane == 0) {
+    if (elect_one()) {
       const uint32_t id = instr_desc(kBM, 128, 1, 1, 0, 1, 0);
       const int npair = args.passes == 3 ? 3 : 1;
       int stage = 0;
@@ -1041,7 +1041,7 @@ k_joint_fwd_tp(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
     }
   } else if (warp == kTpWarpPool) {
     // ------------------------------------------------------------ pooling issuer
-    if (lane == 0) {
+    if (elect_one()) {
       // A = |Z| [128 rows][64 samples] in tensor memory, B = [W_hi ; W_lo] [NP frames][64
       // samples] K-major with 128-byte rows; a K step is 16 samples
       const uint32_t idp = instr_desc(kBM, NP, 1, 1, 0, 0, 0);

@@ -123,7 +123,7 @@ k_joint_bwd_tc(const __grid_constant__ TbMaps maps, TbArgs args, DevPlan P) {
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
-    if (lane == 0) {
+    if (elect_one()) {
       uint32_t a1_ph = 0;
       int wst = 0;
       uint32_t wph = 0;
@@ -170,7 +170,7 @@ k_joint_bwd_tc(const __grid_constant__ TbMaps maps, TbArgs args, DevPlan P) {
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
+    if (elect_one()) {
       const uint32_t t_d1r = tbase, t_d1i = tbase + 32, t_d4 = tbase + 64;
       const uint32_t t_d2r = tbase + 128, t_d2i = tbase + 288;
       uint32_t a1_ph = 0, d1f_ph = 0, d2f_ph = 0;
@@ -437,7 +437,7 @@ k_joint_bwd_tc3(const __grid_constant__ Tb3Maps maps, TbArgs args, DevPlan P) {
   };
 
   if (warp == 0) {
-    if (lane == 0) {
+    if (elect_one()) {
       uint32_t a4_ph = 0, yph = 0, wph = 0;
       int ys = 0, wst = 0;
       int armed_y[2] = {-1, -1}, armed_w[2] = {-1, -1}, armed_a4 = -1;
@@ -490,7 +490,7 @@ k_joint_bwd_tc3(const __grid_constant__ Tb3Maps maps, TbArgs args, DevPlan P) {
       if (armed_a4 >= 0) mbar_wait(&a4_full, (uint32_t)armed_a4, wait_budget);
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (elect_one()) {
       const uint32_t t_d1r = tbase, t_d1i = tbase + 32, t_d4 = tbase + 64;
       const uint32_t t_d2r = tbase + 128, t_d2i = tbase + 288;
       uint32_t a4_ph = 0, d1f_ph = 0, d2f_ph = 0, a2_ph = 0, yph = 0, wph = 0;
@@ -812,7 +812,7 @@ k_joint_bwd_fast(const __grid_constant__ TfMaps maps, TfArgs args, DevPlan P) {
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
-    if (lane == 0) {
+    if (elect_one()) {
       uint32_t a1_ph = 0, wph = 0;
       int wst = 0;
       uint32_t armed_w = 0, armed_w_par = 0;
@@ -863,7 +863,7 @@ k_joint_bwd_fast(const __grid_constant__ TfMaps maps, TfArgs args, DevPlan P) {
   } else if (warp == 1) {
     // ------------------------------------------------------------ first-product issuer
     // Z^T and g|Z|^T of every chunk, up to two chunks ahead of the epilogue
-    if (lane == 0) {
+    if (elect_one()) {
       const uint32_t id1 = instr_desc(128, 2 * RC, 1, 1, 1, 0, 0);
       const uint32_t id4 = instr_desc(128, RC, 1, 1, 0, 0, 0);
       uint32_t a1_ph = 0, wph = 0;
@@ -931,7 +931,7 @@ k_joint_bwd_fast(const __grid_constant__ TfMaps maps, TfArgs args, DevPlan P) {
     // ------------------------------------------------------------ last-product issuer
     // gY^T [Im | Re] += gZi [Wr | Wi] + gZr [-Wi | Wr], chunk by chunk behind the epilogue;
     // releases each W chunk (its first product completed before the epilogue ran)
-    if (lane == 0) {
+    if (elect_one()) {
       const uint32_t id2 = instr_desc(128, 128, 1, 1, 0, 1, 0);
       uint32_t d2f_ph = 0, wph = 0, a2_ph = 0;   // a2_ph bit i: phase of buffer i
       int wst = 0, q2 = 0;
@@ -1181,7 +1181,7 @@ k_joint_bwd_pair(const __grid_constant__ TpMaps maps, TpArgs args, DevPlan P) {
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
-    if (lane == 0) {
+    if (elect_one()) {
       uint32_t a1_ph = 0, wph = 0;
       int wst = 0;
       uint32_t armed_w = 0, armed_w_par = 0;
@@ -1236,7 +1236,7 @@ k_joint_bwd_pair(const __grid_constant__ TpMaps maps, TpArgs args, DevPlan P) {
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ first-product issuer
-    if (lane == 0) {
+    if (elect_one()) {
       const uint32_t id1 = instr_desc(128, 2 * RC, 1, 1, 1, 0, 0);
       const uint32_t id4 = instr_desc(128, 2 * RC, 1, 1, 0, 0, 0);
       uint32_t a1_ph = 0, wph = 0;
@@ -1298,7 +1298,7 @@ k_joint_bwd_pair(const __grid_constant__ TpMaps maps, TpArgs args, DevPlan P) {
     }
   } else if (warp == kFWarpG2) {
     // ------------------------------------------------------------ last-product issuer
-    if (lane == 0) {
+    if (elect_one()) {
       const uint32_t id2 = instr_desc(128, 64 * NAT, 1, 1, 0, 1, 0);
       uint32_t d2f_ph = 0, wph = 0, a2_ph = 0;   // a2_ph bit i: phase of buffer i
       int wst = 0, q2 = 0;
