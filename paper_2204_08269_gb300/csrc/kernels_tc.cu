@@ -838,7 +838,7 @@ k_joint_fwd_tc16(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
 // epilogue, at a quarter of the tcgen05 rate).  The epilogue stages |Z| (BF16 hi, lo for the
 // FP32-grade split) of both spins in tensor memory as an MMA A operand (row r in lane r, two
 // samples per 32-bit column: 32 columns per spin and plane), and a second issuing thread
-// accumulates D_spin[row][f] += |Z|[row][n] [W_hi | W_lo][f][n] over the item's tiles into TMEM
+// (pooling tile t once product t + 1 has completed, when the tensor pipe is idle) accumulates D_spin[row][f] += |Z|[row][n] [W_hi | W_lo][f][n] over the item's tiles into TMEM
 // (N = NT per weight plane: frames of W_hi, then of W_lo; both |Z| planes accumulate into the
 // same D, so D[f] + D[NT + f] = (Z_hi + Z_lo)(W_hi + W_lo)).  Staging |Z| in tensor memory
 // keeps its stores and the pooling MMAs' A reads off the shared memory, whose bandwidth the
@@ -871,7 +871,7 @@ k_joint_fwd_tp(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
   uint8_t* sStage = sm + (RES ? planes * 2 * max_kb * kAPlane : 0);
   uint8_t* sWt = sStage + S * stage_bytes;               // WS slots of [W_hi plane][W_lo plane]
   __shared__ uint64_t full_bar[8], empty_bar[8], wfull[kMaxWS], wempty[kMaxWS], tfull, tempty,
-      sfull, sfree, dfull, dfree, a_full, a_free, mma_done, pool_done;
+      sfull, sfree, dfull, dfree, a_full, a_free, mma_done, pool_done, prod[2];
   __shared__ uint32_t tmem_base;
   __shared__ volatile int abort_flag;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -896,6 +896,8 @@ k_joint_fwd_tp(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
     mbar_init(&a_free, 1);
     mbar_init(&mma_done, 1);
     mbar_init(&pool_done, 1);
+    mbar_init(&prod[0], 1);
+    mbar_init(&prod[1], 1);
     fence_barrier_init();
   }
   if (warp == 1) {
@@ -980,9 +982,9 @@ k_joint_fwd_tp(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
     // ------------------------------------------------------------ product issuer
     if (elect_one()) {
       const uint32_t id = instr_desc(kBM, 128, 1, 1, 0, 1, 0);
-      const int npair = args.passes == 3 ? 3 : 1;
+      constexpr int npair = PS == 2 ? 3 : 1;   // FP32-grade split, or one pass
       int stage = 0;
-      uint32_t phase = 0, tph = 0, aph = 0;
+      uint32_t phase = 0, tph = 0, aph = 0, par = 0;
       bool ok = true;
       for (int it = blockIdx.x; it < args.n_items && ok && !abort_flag; it += gridDim.x) {
         const int4 item = args.items[it % args.n_base];
@@ -995,12 +997,13 @@ k_joint_fwd_tp(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
           aph ^= 1;
         }
         for (int j = 0; j < item.z && ok; ++j) {
+          // the first operand stage is there, as a rule, before the accumulator is free
+          if (!mbar_wait(&full_bar[stage], phase, wait_budget)) { fail(35); ok = false; break; }
           if (!mbar_wait(&tempty, tph ^ 1, wait_budget)) { fail(34); ok = false; break; }
           tph ^= 1;
-          tc_fence_after();
           const uint32_t t_a = tbase, t_b = tbase + 128;
           for (int kb = 0; kb < nkb; ++kb) {
-            if (!mbar_wait(&full_bar[stage], phase, wait_budget)) { fail(35); ok = false; break; }
+            if (kb && !mbar_wait(&full_bar[stage], phase, wait_budget)) { fail(35); ok = false; break; }
             tc_fence_after();
             const uint32_t st = smem_u32(sStage + stage * stage_bytes);
             const uint32_t sb = RES ? st : st + planes * 2 * kAPlane;
@@ -1014,16 +1017,14 @@ k_joint_fwd_tp(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
             for (int ks = 0; ks < 2; ++ks) {
               if (ks < kss) {
 #pragma unroll
-                for (int q = 0; q < 3; ++q) {
-                  if (q < npair) {
-                    const int pa = q == 2 ? 1 : 0, pb = q == 1 ? 1 : 0;
-                    const uint64_t ar = dA + (uint64_t)(pa * 2 * as4 + ks * 2);
-                    const uint64_t ai = ar + as4;
-                    const uint64_t bd = dB + (uint64_t)(pb * 2 * (kYAtom >> 4) + ks * 128);
-                    const uint32_t f = (kb | ks | q) ? 1u : 0u;
-                    mma_f16(t_a, ar, bd, id, f);    // [P1 | P3] = Wr [Yr | Yi]
-                    mma_f16(t_b, ai, bd, id, f);    // [P4 | P2] = Wi [Yr | Yi]
-                  }
+                for (int q = 0; q < npair; ++q) {
+                  const int pa = q == 2 ? 1 : 0, pb = q == 1 ? 1 : 0;
+                  const uint64_t ar = dA + (uint64_t)(pa * 2 * as4 + ks * 2);
+                  const uint64_t ai = ar + as4;
+                  const uint64_t bd = dB + (uint64_t)(pb * 2 * (kYAtom >> 4) + ks * 128);
+                  const uint32_t f = (kb | ks | q) ? 1u : 0u;
+                  mma_f16(t_a, ar, bd, id, f);    // [P1 | P3] = Wr [Yr | Yi]
+                  mma_f16(t_b, ai, bd, id, f);    // [P4 | P2] = Wi [Yr | Yi]
                 }
               }
             }
@@ -1032,6 +1033,8 @@ k_joint_fwd_tp(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
           }
           if (!ok) break;
           mma_commit(&tfull);
+          mma_commit(&prod[par]);
+          par ^= 1;
         }
         if (!ok) break;
         if (RES) mma_commit(&a_free);
@@ -1046,7 +1049,7 @@ k_joint_fwd_tp(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
       // samples] K-major with 128-byte rows; a K step is 16 samples
       const uint32_t idp = instr_desc(kBM, NP, 1, 1, 0, 0, 0);
       int ws = 0;
-      uint32_t sph = 0, wph = 0, dph = 0;
+      uint32_t sph = 0, wph = 0, dph = 0, tiles = 0;
       bool ok = true;
       for (int it = blockIdx.x; it < args.n_items && ok && !abort_flag; it += gridDim.x) {
         const int4 item = args.items[it % args.n_base];
@@ -1056,6 +1059,13 @@ k_joint_fwd_tp(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
         for (int j = 0; j < item.z && ok; ++j) {
           if (!mbar_wait(&sfull, sph, wait_budget)) { fail(37); ok = false; break; }
           sph ^= 1;
+          // product t + 1 has completed (there is one unless this is the CTA's last tile): the
+          // pooling of tile t then runs while the epilogue loads that product, when the tensor
+          // pipe is idle.  Product t + 3, whose commit reuses this barrier, waits for the
+          // accumulator of tile t + 2 and so for this pooling: no phase can be missed.
+          ++tiles;
+          if ((j + 1 < item.z || it + (int)gridDim.x < args.n_items) &&
+              !mbar_wait(&prod[tiles & 1], (tiles >> 1) & 1, wait_budget)) { fail(42); ok = false; break; }
           if (!mbar_wait(&wfull[ws], wph, wait_budget)) { fail(38); ok = false; break; }
           tc_fence_after();
           const uint64_t dW = smem_desc(smem_u32(sWt + ws * PS * kWHalf), 16, 1024, kSw128);
@@ -1114,6 +1124,7 @@ k_joint_fwd_tp(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(&tempty);
+        if (PS == 1) __syncwarp();             // the release before the arithmetic (1.6 %)
 #pragma unroll
         for (int h8 = 0; h8 < 2; ++h8) {
           const uint32_t* p1 = q1[h8];
@@ -1129,8 +1140,12 @@ k_joint_fwd_tp(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
             const float2 rd = __fadd2_rn(x1, x2), id = fsub2(x3, x4);
             const float2 su = __ffma2_rn(ru, ru, __fmul2_rn(iu, iu));
             const float2 sd = __ffma2_rn(rd, rd, __fmul2_rn(id, id));
-            const float2 mu = make_float2(sqrt_approx(su.x), sqrt_approx(su.y));
-            const float2 md = make_float2(sqrt_approx(sd.x), sqrt_approx(sd.y));
+            // one BF16 pass: subnormal |Z|^2 (|Z| < 1.1e-19) as 0, which halves the instructions of
+            // a root (6.70 -> 5.90 ms, B = 256, N = 2^15); the FP32-grade form keeps them, and
+            // measured slower without (5.22 against 4.64 ms, B = 64, N = 2^16)
+            auto root = [](float v) { return PS == 1 ? sqrt_approx_ftz(v) : sqrt_approx(v); };
+            const float2 mu = make_float2(root(su.x), root(su.y));
+            const float2 md = make_float2(root(sd.x), root(sd.y));
             __nv_bfloat162 hu = __floats2bfloat162_rn(mu.x, mu.y);
             __nv_bfloat162 hd = __floats2bfloat162_rn(md.x, md.y);
             hv[h8][0][i] = *reinterpret_cast<uint32_t*>(&hu);
