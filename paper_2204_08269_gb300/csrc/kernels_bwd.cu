@@ -23,6 +23,7 @@ namespace {
 
 __global__ void __launch_bounds__(kFftThreads)
 k_uh_from_u1(DevPlan P, const float* __restrict__ u1, float2* __restrict__ uh) {
+  pdl_enter();
   extern __shared__ float2 sm[];
   const int lam = blockIdx.x, b = blockIdx.y;
   const Row1 R = P.rows1[lam];
@@ -75,6 +76,7 @@ template <int NC>
 __global__ void __launch_bounds__(kJT)
 k_joint_bwd_simt(DevPlan P, const int2* __restrict__ items, const float2* __restrict__ y,
                  const float* __restrict__ gs2, float2* __restrict__ gy) {
+  pdl_enter();
   extern __shared__ float4 smraw[];
   float* smf = reinterpret_cast<float*>(smraw);
   const int2 it = items[blockIdx.x];
@@ -247,6 +249,7 @@ k_joint_bwd_simt(DevPlan P, const int2* __restrict__ items, const float2* __rest
 // order.
 __global__ void __launch_bounds__(kRowBound)
 k_gy_spectra(DevPlan P, const int4* __restrict__ items, float2* __restrict__ gy) {
+  pdl_enter();
   extern __shared__ float2 sm[];
   const int4 it = items[blockIdx.x];
   const int a = it.x, lam0 = it.y, G = it.z, b = blockIdx.y;
@@ -313,6 +316,7 @@ k_gy_spectra(DevPlan P, const int4* __restrict__ items, float2* __restrict__ gy)
 __global__ void __launch_bounds__(256, 3)   // launched with 256 threads; three blocks per SM
 k_second_order_bwd(DevPlan P, const float2* __restrict__ gys, const float* __restrict__ gs1,
                    float* __restrict__ gu1) {
+  pdl_enter();
   extern __shared__ float2 sm[];
   const int lam = blockIdx.x, b = blockIdx.y;
   const Row1 R = P.rows1[lam];
@@ -388,6 +392,7 @@ k_second_order_bwd(DevPlan P, const float2* __restrict__ gys, const float* __res
 __global__ void __launch_bounds__(kRowLaunch, 3)   // three 256-thread blocks per SM
 k_stage1_bwd(DevPlan P, const float2* __restrict__ xh, const float* __restrict__ gu1,
              float2* __restrict__ gf) {
+  pdl_enter();
   extern __shared__ float2 sm[];
   const int lam = blockIdx.x, b = blockIdx.y;
   const Row1 R = P.rows1[lam];
@@ -422,6 +427,7 @@ k_stage1_bwd(DevPlan P, const float2* __restrict__ xh, const float* __restrict__
 // phi-hat reaches the Nyquist bin (T <= 2), k_gx adds it in the time domain instead.
 __global__ void k_gxh(DevPlan P, const float2* __restrict__ gf, const float* __restrict__ gs0,
                       float2* __restrict__ gxh) {
+  pdl_enter();
   const int b = blockIdx.y;
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   const int half = P.N >> 1;
@@ -461,6 +467,7 @@ __global__ void k_gxh(DevPlan P, const float2* __restrict__ gf, const float* __r
 // (S0's adjoint is already in H unless phi-hat reaches the Nyquist bin)
 __global__ void __launch_bounds__(kFftThreads, 2)   // two 512-thread blocks per SM
 k_gx(DevPlan P, const float2* __restrict__ gxh, const float* __restrict__ gs0, float* __restrict__ gx) {
+  pdl_enter();
   extern __shared__ float2 sm[];
   const int r = blockIdx.x, b = blockIdx.y;
   const int half = P.N >> 1;
@@ -503,6 +510,7 @@ template <int FB>
 __global__ void __launch_bounds__(kRowBound)
 k_scat1d_bwd_rows(DevPlan P, const int4* __restrict__ items, const float2* __restrict__ uh,
                   const float* __restrict__ gs2t, float2* __restrict__ gy) {
+  pdl_enter();
   extern __shared__ float2 sm[];
   __shared__ int s_off[kMaxRowsPerItem], s_kend[kMaxRowsPerItem];
   __shared__ float s_inv[kMaxRowsPerItem];
@@ -594,8 +602,7 @@ static void launch_joint_bwd_simt(const jtfs_plan* p, int n_items, const int* it
   const bool wide = (size_t)w.total * 4 <= 227 * 1024;
   const JointBwdLayout l = wide ? w : joint_bwd_layout(p->n1, p->n_t, 16);
   auto* kernel = wide ? k_joint_bwd_simt<32> : k_joint_bwd_simt<16>;
-  kernel<<<dim3((unsigned)n_items, B, wide ? 1 : 2), l.threads, (size_t)l.total * 4, st>>>(
-      p->dp, reinterpret_cast<const int2*>(items), y, gs2, gy);
+  launch_pdl(kernel, dim3((unsigned)n_items, B, wide ? 1 : 2), l.threads, (size_t)l.total * 4, st, p->dp, reinterpret_cast<const int2*>(items), y, gs2, gy);
 }
 
 bool backward_reuses_forward(const jtfs_plan* p) {
@@ -616,22 +623,19 @@ jtfs_status launch_backward(const jtfs_plan* p, const float* x, const float* u1,
   if (!fused) {
     {
       StageScope sc(p, kStXfft, st, 2);
-      k_xfft_sub<<<dim3(d.D, B), kFftThreads, (size_t)d.M * 17 / 2, st>>>(d, x, w.xsub);
-      k_xfft_combine<<<dim3((p->N / 2 + 255) / 256, B), 256, 0, st>>>(d, w.xsub, w.xh);
+      launch_pdl(k_xfft_sub, dim3(d.D, B), kFftThreads, (size_t)d.M * 17 / 2, st, d, x, w.xsub);
+      launch_pdl(k_xfft_combine, dim3((p->N / 2 + 255) / 256, B), 256, 0, st, d, w.xsub, w.xh);
     }
     {
       StageScope sc(p, kStUhFromU1, st, 1);
-      k_uh_from_u1<<<dim3(p->n1, B), kFftThreads, (size_t)p->L1max * 17 / 2, st>>>(d, u1, w.uh);
+      launch_pdl(k_uh_from_u1, dim3(p->n1, B), kFftThreads, (size_t)p->L1max * 17 / 2, st, d, u1, w.uh);
     }
   }
   const size_t n_items = p->items.size() / 2;
   if (gs2 && n_items > 0 && p->use_tcb) {
     if (!reuse_y) {
       StageScope sc(p, kStSecondOrder, st, 1);
-      k_second_order_rows<1><<<dim3((unsigned)(p->rowitems.size() / 4), B), p->row_threads,
-                              (size_t)p->rows_cap * 17 / 2, st>>>(
-          d, reinterpret_cast<const int4*>(p->d_rowitems), w.uh, nullptr,
-          (__nv_bfloat16*)w.ybh, (__nv_bfloat16*)w.ybl, B);
+      launch_pdl(k_second_order_rows<1>, dim3((unsigned)(p->rowitems.size() / 4), B), p->row_threads, (size_t)p->rows_cap * 17 / 2, st, d, reinterpret_cast<const int4*>(p->d_rowitems), w.uh, nullptr, (__nv_bfloat16*)w.ybh, (__nv_bfloat16*)w.ybl, B);
     }
     StageScope sc(p, kStJointBwd, st, 0);   // the launcher counts its kernels
     jtfs_status r2 = launch_joint_bwd_tc(p, B, w.ybh, w.ybl, gs2, w.g1, w.gy, st);
@@ -639,10 +643,7 @@ jtfs_status launch_backward(const jtfs_plan* p, const float* x, const float* u1,
     if (!p->tcb_fb_items.empty()) {
       // rates beyond the tensor-core backward's lambda' capacity: FP32 Y rows of those rates
       // only, then the CUDA-core backward on them
-      k_second_order_rows<0><<<dim3((unsigned)(p->tcb_fb_rowitems.size() / 4), B),
-                              p->row_threads, (size_t)p->tcb_fb_cap * 17 / 2, st>>>(
-          d, reinterpret_cast<const int4*>(p->d_tcb_fb_rowitems), w.uh, w.y, nullptr, nullptr,
-          B);
+      launch_pdl(k_second_order_rows<0>, dim3((unsigned)(p->tcb_fb_rowitems.size() / 4), B), p->row_threads, (size_t)p->tcb_fb_cap * 17 / 2, st, d, reinterpret_cast<const int4*>(p->d_tcb_fb_rowitems), w.uh, w.y, nullptr, nullptr, B);
       launch_joint_bwd_simt(p, (int)(p->tcb_fb_items.size() / 2), p->d_tcb_fb_items, B, w.y, gs2,
                             w.gy, st);
       p->prof.launches += 2;
@@ -650,9 +651,7 @@ jtfs_status launch_backward(const jtfs_plan* p, const float* x, const float* u1,
   } else if (gs2 && n_items > 0) {
     {
       StageScope sc(p, kStSecondOrder, st, 1);
-      k_second_order_rows<0><<<dim3((unsigned)(p->rowitems.size() / 4), B), p->row_threads,
-                              (size_t)p->rows_cap * 17 / 2, st>>>(
-          d, reinterpret_cast<const int4*>(p->d_rowitems), w.uh, w.y, nullptr, nullptr, B);
+      launch_pdl(k_second_order_rows<0>, dim3((unsigned)(p->rowitems.size() / 4), B), p->row_threads, (size_t)p->rows_cap * 17 / 2, st, d, reinterpret_cast<const int4*>(p->d_rowitems), w.uh, w.y, nullptr, nullptr, B);
     }
     StageScope sc(p, kStJointBwd, st, 1);
     launch_joint_bwd_simt(p, (int)n_items, p->d_items, B, w.y, gs2, w.gy, st);
@@ -662,19 +661,17 @@ jtfs_status launch_backward(const jtfs_plan* p, const float* x, const float* u1,
   {
     StageScope sc(p, kStSecondOrderBwd, st, 2);
     if (!p->rowitems.empty())
-      k_gy_spectra<<<dim3((unsigned)(p->rowitems.size() / 4), B), p->row_threads,
-                     (size_t)p->rows_cap * 17 / 2, st>>>(
-          d, reinterpret_cast<const int4*>(p->d_rowitems), w.gy);
-    k_second_order_bwd<<<dim3(p->n1, B), 256, (size_t)p->L1max * 17 / 2, st>>>(d, w.gy, gs1, w.gu1);
+      launch_pdl(k_gy_spectra, dim3((unsigned)(p->rowitems.size() / 4), B), p->row_threads, (size_t)p->rows_cap * 17 / 2, st, d, reinterpret_cast<const int4*>(p->d_rowitems), w.gy);
+    launch_pdl(k_second_order_bwd, dim3(p->n1, B), 256, (size_t)p->L1max * 17 / 2, st, d, w.gy, gs1, w.gu1);
   }
   {
     StageScope sc(p, kStStage1Bwd, st, 1);
-    k_stage1_bwd<<<dim3(p->n1, B), kRowLaunch, (size_t)p->L1max * 17 / 2, st>>>(d, w.xh, w.gu1, w.gf);
+    launch_pdl(k_stage1_bwd, dim3(p->n1, B), kRowLaunch, (size_t)p->L1max * 17 / 2, st, d, w.xh, w.gu1, w.gf);
   }
   {
     StageScope sc(p, kStGx, st, 2);
-    k_gxh<<<dim3((p->N / 2 + 255) / 256, B), 256, 0, st>>>(d, w.gf, gs0, w.gxh);
-    k_gx<<<dim3(d.D, B), kFftThreads, (size_t)d.M * 17 / 2, st>>>(d, w.gxh, gs0, gx);
+    launch_pdl(k_gxh, dim3((p->N / 2 + 255) / 256, B), 256, 0, st, d, w.gf, gs0, w.gxh);
+    launch_pdl(k_gx, dim3(d.D, B), kFftThreads, (size_t)d.M * 17 / 2, st, d, w.gxh, gs0, gx);
   }
   return cuda_check(cudaGetLastError(), "backward launch");
 }
@@ -689,40 +686,36 @@ jtfs_status launch_scat1d_backward(const jtfs_plan* p, const float* x, const flo
   const DevPlan& d = p->dp;
   {
     StageScope sc(p, kStXfft, st, 2);
-    k_xfft_sub<<<dim3(d.D, B), kFftThreads, (size_t)d.M * 17 / 2, st>>>(d, x, w.xsub);
-    k_xfft_combine<<<dim3((p->N / 2 + 255) / 256, B), 256, 0, st>>>(d, w.xsub, w.xh);
+    launch_pdl(k_xfft_sub, dim3(d.D, B), kFftThreads, (size_t)d.M * 17 / 2, st, d, x, w.xsub);
+    launch_pdl(k_xfft_combine, dim3((p->N / 2 + 255) / 256, B), 256, 0, st, d, w.xsub, w.xh);
   }
   {
     StageScope sc(p, kStUhFromU1, st, 1);
-    k_uh_from_u1<<<dim3(p->n1, B), kFftThreads, (size_t)p->L1max * 17 / 2, st>>>(d, u1, w.uh);
+    launch_pdl(k_uh_from_u1, dim3(p->n1, B), kFftThreads, (size_t)p->L1max * 17 / 2, st, d, u1, w.uh);
   }
   if (gs2t && !p->rowitems.empty()) {
     StageScope sc(p, kStJointBwd, st, 1);
     auto* kernel = p->n_t >= 8 ? k_scat1d_bwd_rows<8>
                    : p->n_t == 4 ? k_scat1d_bwd_rows<4>
                    : p->n_t == 2 ? k_scat1d_bwd_rows<2> : k_scat1d_bwd_rows<1>;
-    kernel<<<dim3((unsigned)(p->rowitems.size() / 4), B), p->row_threads,
-             (size_t)p->rows_cap * 17 / 2, st>>>(
-        d, reinterpret_cast<const int4*>(p->d_rowitems), w.uh, gs2t, w.gy);
+    launch_pdl(kernel, dim3((unsigned)(p->rowitems.size() / 4), B), p->row_threads, (size_t)p->rows_cap * 17 / 2, st, d, reinterpret_cast<const int4*>(p->d_rowitems), w.uh, gs2t, w.gy);
   } else if (p->y_len > 0) {
     cudaMemsetAsync(w.gy, 0, (size_t)B * p->y_len * sizeof(float2), st);
   }
   {
     StageScope sc(p, kStSecondOrderBwd, st, 2);
     if (!p->rowitems.empty())
-      k_gy_spectra<<<dim3((unsigned)(p->rowitems.size() / 4), B), p->row_threads,
-                     (size_t)p->rows_cap * 17 / 2, st>>>(
-          d, reinterpret_cast<const int4*>(p->d_rowitems), w.gy);
-    k_second_order_bwd<<<dim3(p->n1, B), 256, (size_t)p->L1max * 17 / 2, st>>>(d, w.gy, gs1, w.gu1);
+      launch_pdl(k_gy_spectra, dim3((unsigned)(p->rowitems.size() / 4), B), p->row_threads, (size_t)p->rows_cap * 17 / 2, st, d, reinterpret_cast<const int4*>(p->d_rowitems), w.gy);
+    launch_pdl(k_second_order_bwd, dim3(p->n1, B), 256, (size_t)p->L1max * 17 / 2, st, d, w.gy, gs1, w.gu1);
   }
   {
     StageScope sc(p, kStStage1Bwd, st, 1);
-    k_stage1_bwd<<<dim3(p->n1, B), kRowLaunch, (size_t)p->L1max * 17 / 2, st>>>(d, w.xh, w.gu1, w.gf);
+    launch_pdl(k_stage1_bwd, dim3(p->n1, B), kRowLaunch, (size_t)p->L1max * 17 / 2, st, d, w.xh, w.gu1, w.gf);
   }
   {
     StageScope sc(p, kStGx, st, 2);
-    k_gxh<<<dim3((p->N / 2 + 255) / 256, B), 256, 0, st>>>(d, w.gf, gs0, w.gxh);
-    k_gx<<<dim3(d.D, B), kFftThreads, (size_t)d.M * 17 / 2, st>>>(d, w.gxh, gs0, gx);
+    launch_pdl(k_gxh, dim3((p->N / 2 + 255) / 256, B), 256, 0, st, d, w.gf, gs0, w.gxh);
+    launch_pdl(k_gx, dim3(d.D, B), kFftThreads, (size_t)d.M * 17 / 2, st, d, w.gxh, gs0, gx);
   }
   return cuda_check(cudaGetLastError(), "time scattering backward");
 }

@@ -39,6 +39,7 @@ constexpr int kS0Split = 8, kS0Threads = 256;
 
 __global__ void __cluster_dims__(kS0Split, 1, 1) __launch_bounds__(kS0Threads)
 k_s0(DevPlan P, const float* __restrict__ x, float* __restrict__ s0) {
+  pdl_enter();
   __shared__ double red[kS0Threads / 32];
   __shared__ double parts[kS0Split];
   cg::cluster_group cl = cg::this_cluster();
@@ -79,6 +80,7 @@ k_s0(DevPlan P, const float* __restrict__ x, float* __restrict__ s0) {
 __global__ void __launch_bounds__(kRowLaunch, 3)   // three 256-thread blocks per SM
 k_scalogram(DevPlan P, const float2* __restrict__ xh, float* __restrict__ u1,
             float2* __restrict__ uh, float* __restrict__ s1) {
+  pdl_enter();
   extern __shared__ float2 sm[];
   const int lam = blockIdx.x, b = blockIdx.y;
   const Row1 R = P.rows1[lam];
@@ -152,6 +154,7 @@ struct JointSmem {
 
 __global__ void __launch_bounds__(kJT)
 k_joint_fwd_simt(DevPlan P, const float2* __restrict__ y, float* __restrict__ s2) {
+  pdl_enter();
   extern __shared__ float4 smraw[];
   const int c = blockIdx.x, a = blockIdx.y, b = blockIdx.z;
   const Rate2 A = P.rates2[a];
@@ -258,6 +261,7 @@ k_joint_fwd_simt(DevPlan P, const float2* __restrict__ y, float* __restrict__ s2
 // through shared memory; grid (ceil(L / 32), ceil(kt / 32), 2 B) for one rate.
 __global__ void k_transpose_yt(DevPlan P, int a, const float* __restrict__ y,
                                float* __restrict__ yt, int B) {
+  pdl_enter();
   __shared__ float tile[32][33];
   const Rate2 A = P.rates2[a];
   const int lm8 = A.lam_min & ~7;
@@ -349,6 +353,7 @@ template <int FB>
 __global__ void __launch_bounds__(kRowThreads)
 k_scat1d_rows(DevPlan P, const int4* __restrict__ items, const float2* __restrict__ uh,
               float* __restrict__ s2t) {
+  pdl_enter();
   extern __shared__ float2 sm[];
   // the row tables, then (once the moduli are taken) the partials of shared rows: one array, so
   // that three 256-thread blocks still fit an SM
@@ -475,12 +480,9 @@ jtfs_status autotune_rows(jtfs_plan* p, int B, const Workspace& w, cudaStream_t 
         const dim3 grid((unsigned)(items.size() / 4), B);
         const size_t smem = (size_t)caps[ci] * 17 / 2;   // padded one per 16
         if (p->use_tc)
-          k_second_order_rows<1><<<grid, threads, smem, st>>>(
-              d, reinterpret_cast<const int4*>(d_items), w.uh, nullptr, (__nv_bfloat16*)w.ybh,
-              (__nv_bfloat16*)w.ybl, B);
+          launch_pdl(k_second_order_rows<1>, grid, threads, smem, st, d, reinterpret_cast<const int4*>(d_items), w.uh, nullptr, (__nv_bfloat16*)w.ybh, (__nv_bfloat16*)w.ybl, B);
         else
-          k_second_order_rows<0><<<grid, threads, smem, st>>>(
-              d, reinterpret_cast<const int4*>(d_items), w.uh, w.y, nullptr, nullptr, B);
+          launch_pdl(k_second_order_rows<0>, grid, threads, smem, st, d, reinterpret_cast<const int4*>(d_items), w.uh, w.y, nullptr, nullptr, B);
       };
       launch();
       cudaEventRecord(e0, st);
@@ -524,16 +526,16 @@ jtfs_status launch_scat1d_forward(const jtfs_plan* p, const float* x, int B, flo
   const DevPlan& d = p->dp;
   {
     StageScope sc(p, kStXfft, st, 2);
-    k_xfft_sub<<<dim3(d.D, B), kFftThreads, (size_t)d.M * 17 / 2, st>>>(d, x, w.xsub);
-    k_xfft_combine<<<dim3((p->N / 2 + 255) / 256, B), 256, 0, st>>>(d, w.xsub, w.xh);
+    launch_pdl(k_xfft_sub, dim3(d.D, B), kFftThreads, (size_t)d.M * 17 / 2, st, d, x, w.xsub);
+    launch_pdl(k_xfft_combine, dim3((p->N / 2 + 255) / 256, B), 256, 0, st, d, w.xsub, w.xh);
   }
   {
     StageScope sc(p, kStS0, st, 1);
-    k_s0<<<dim3(kS0Split * p->n_t, B), kS0Threads, 0, st>>>(d, x, s0);
+    launch_pdl(k_s0, dim3(kS0Split * p->n_t, B), kS0Threads, 0, st, d, x, s0);
   }
   {
     StageScope sc(p, kStScalogram, st, 1);
-    k_scalogram<<<dim3(p->n1, B), kRowLaunch, (size_t)p->L1max * 17 / 2 + (size_t)p->L1max * 4, st>>>(d, w.xh, u1, w.uh, s1);
+    launch_pdl(k_scalogram, dim3(p->n1, B), kRowLaunch, (size_t)p->L1max * 17 / 2 + (size_t)p->L1max * 4, st, d, w.xh, u1, w.uh, s1);
   }
   if ((rc = cuda_check(cudaMemsetAsync(s2t, 0, (size_t)B * p->n2 * p->n1 * p->n_t * sizeof(float), st), "memset")) != JTFS_OK)
     return rc;
@@ -543,9 +545,7 @@ jtfs_status launch_scat1d_forward(const jtfs_plan* p, const float* x, int B, flo
     auto* kernel = p->n_t >= 8 ? k_scat1d_rows<8>
                    : p->n_t == 4 ? k_scat1d_rows<4>
                    : p->n_t == 2 ? k_scat1d_rows<2> : k_scat1d_rows<1>;
-    kernel<<<dim3((unsigned)(p->rowitems.size() / 4), B), p->row_threads,
-             (size_t)p->rows_cap * 17 / 2, st>>>(
-        d, reinterpret_cast<const int4*>(p->d_rowitems), w.uh, s2t);
+    launch_pdl(kernel, dim3((unsigned)(p->rowitems.size() / 4), B), p->row_threads, (size_t)p->rows_cap * 17 / 2, st, d, reinterpret_cast<const int4*>(p->d_rowitems), w.uh, s2t);
   }
   return cuda_check(cudaGetLastError(), "time scattering forward");
 }
@@ -557,32 +557,29 @@ jtfs_status launch_forward(const jtfs_plan* p, const float* x, int B, float* s0,
   const DevPlan& d = p->dp;
   {
     StageScope sc(p, kStXfft, st, 2);
-    k_xfft_sub<<<dim3(d.D, B), kFftThreads, (size_t)d.M * 17 / 2, st>>>(d, x, w.xsub);
-    k_xfft_combine<<<dim3((p->N / 2 + 255) / 256, B), 256, 0, st>>>(d, w.xsub, w.xh);
+    launch_pdl(k_xfft_sub, dim3(d.D, B), kFftThreads, (size_t)d.M * 17 / 2, st, d, x, w.xsub);
+    launch_pdl(k_xfft_combine, dim3((p->N / 2 + 255) / 256, B), 256, 0, st, d, w.xsub, w.xh);
   }
   {
     StageScope sc(p, kStS0, st, 1);
-    k_s0<<<dim3(kS0Split * p->n_t, B), kS0Threads, 0, st>>>(d, x, s0);
+    launch_pdl(k_s0, dim3(kS0Split * p->n_t, B), kS0Threads, 0, st, d, x, s0);
   }
   {
     StageScope sc(p, kStScalogram, st, 1);
-    k_scalogram<<<dim3(p->n1, B), kRowLaunch, (size_t)p->L1max * 17 / 2 + (size_t)p->L1max * 4, st>>>(d, w.xh, u1, w.uh, s1);
+    launch_pdl(k_scalogram, dim3(p->n1, B), kRowLaunch, (size_t)p->L1max * 17 / 2 + (size_t)p->L1max * 4, st, d, w.xh, u1, w.uh, s1);
   }
   if (p->use_tc && p->cfg.precision == JTFS_PREC_TF32) {
     // TF32 operands: Y as FP32 planes (in the complex FP32 buffer, same size)
     if (!p->pairs.empty()) {
       StageScope sc(p, kStSecondOrder, st, 1);
-      k_second_order_rows<2><<<dim3((unsigned)(p->rowitems.size() / 4), B), p->row_threads,
-                              (size_t)p->rows_cap * 17 / 2, st>>>(
-          d, reinterpret_cast<const int4*>(p->d_rowitems), w.uh, w.y, nullptr, nullptr, B);
+      launch_pdl(k_second_order_rows<2>, dim3((unsigned)(p->rowitems.size() / 4), B), p->row_threads, (size_t)p->rows_cap * 17 / 2, st, d, reinterpret_cast<const int4*>(p->d_rowitems), w.uh, w.y, nullptr, nullptr, B);
     }
     {
       StageScope sc(p, kStSecondOrder, st, 0);
       for (int a = 0; a < p->n2; ++a) {
         const Rate2& A = p->rates2[a];
         if (A.s == 0 || A.kt == 0) continue;
-        k_transpose_yt<<<dim3((A.L + 31) / 32, (A.kt + 31) / 32, 2 * B), dim3(32, 8), 0, st>>>(
-            d, a, reinterpret_cast<const float*>(w.y), w.yt, B);
+        launch_pdl(k_transpose_yt, dim3((A.L + 31) / 32, (A.kt + 31) / 32, 2 * B), dim3(32, 8), 0, st, d, a, reinterpret_cast<const float*>(w.y), w.yt, B);
         ++p->prof.launches;
       }
     }
@@ -592,10 +589,7 @@ jtfs_status launch_forward(const jtfs_plan* p, const float* x, int B, float* s0,
   } else if (p->use_tc) {
     if (!p->pairs.empty()) {
       StageScope sc(p, kStSecondOrder, st, 1);
-      k_second_order_rows<1><<<dim3((unsigned)(p->rowitems.size() / 4), B), p->row_threads,
-                              (size_t)p->rows_cap * 17 / 2, st>>>(
-          d, reinterpret_cast<const int4*>(p->d_rowitems), w.uh, nullptr,
-          (__nv_bfloat16*)w.ybh, (__nv_bfloat16*)w.ybl, B);
+      launch_pdl(k_second_order_rows<1>, dim3((unsigned)(p->rowitems.size() / 4), B), p->row_threads, (size_t)p->rows_cap * 17 / 2, st, d, reinterpret_cast<const int4*>(p->d_rowitems), w.uh, nullptr, (__nv_bfloat16*)w.ybh, (__nv_bfloat16*)w.ybl, B);
     }
     StageScope sc(p, kStJointFwd, st, 0);   // the launcher counts its kernels
     jtfs_status r2 = launch_joint_fwd_tc(p, B, w.ybh, w.ybl, w.pbuf, s2, st);
@@ -603,12 +597,10 @@ jtfs_status launch_forward(const jtfs_plan* p, const float* x, int B, float* s0,
   } else {
     if (!p->pairs.empty()) {
       StageScope sc(p, kStSecondOrder, st, 1);
-      k_second_order_rows<0><<<dim3((unsigned)(p->rowitems.size() / 4), B), p->row_threads,
-                              (size_t)p->rows_cap * 17 / 2, st>>>(
-          d, reinterpret_cast<const int4*>(p->d_rowitems), w.uh, w.y, nullptr, nullptr, B);
+      launch_pdl(k_second_order_rows<0>, dim3((unsigned)(p->rowitems.size() / 4), B), p->row_threads, (size_t)p->rows_cap * 17 / 2, st, d, reinterpret_cast<const int4*>(p->d_rowitems), w.uh, w.y, nullptr, nullptr, B);
     }
     StageScope sc(p, kStJointFwd, st, 1);
-    k_joint_fwd_simt<<<dim3(p->C, p->n2, B), kJT, joint_fwd_smem(p), st>>>(d, w.y, s2);
+    launch_pdl(k_joint_fwd_simt, dim3(p->C, p->n2, B), kJT, joint_fwd_smem(p), st, d, w.y, s2);
   }
   return cuda_check(cudaGetLastError(), "forward launch");
 }
@@ -686,10 +678,10 @@ jtfs_status launch_first_order_static(const jtfs_plan* p, const float* x, int B,
   c += a(Bz * p->u1_len * 4);
   float2* uh = (float2*)c;
   const DevPlan& d = p->dp;
-  k_xfft_sub<<<dim3(d.D, B), kFftThreads, (size_t)d.M * 17 / 2, st>>>(d, x, xsub);
-  k_xfft_combine<<<dim3((p->N / 2 + 255) / 256, B), 256, 0, st>>>(d, xsub, xh);
-  k_s0<<<dim3(kS0Split * p->n_t, B), kS0Threads, 0, st>>>(d, x, s0);
-  k_scalogram<<<dim3(p->n1, B), kRowLaunch, (size_t)p->L1max * 17 / 2 + (size_t)p->L1max * 4, st>>>(d, xh, u1, uh, s1);
+  launch_pdl(k_xfft_sub, dim3(d.D, B), kFftThreads, (size_t)d.M * 17 / 2, st, d, x, xsub);
+  launch_pdl(k_xfft_combine, dim3((p->N / 2 + 255) / 256, B), 256, 0, st, d, xsub, xh);
+  launch_pdl(k_s0, dim3(kS0Split * p->n_t, B), kS0Threads, 0, st, d, x, s0);
+  launch_pdl(k_scalogram, dim3(p->n1, B), kRowLaunch, (size_t)p->L1max * 17 / 2 + (size_t)p->L1max * 4, st, d, xh, u1, uh, s1);
   return cuda_check(cudaGetLastError(), "first-order static launch");
 }
 

@@ -29,6 +29,7 @@
 
 #include "fft.cuh"
 #include "internal.h"
+#include "pdl.cuh"
 #include "tma_host.h"
 #include "umma.cuh"
 
@@ -65,6 +66,7 @@ struct TcArgs {
   int nt;                  // frames
   float* P;                // [B][n2][C*n1][nt]
   int n2;
+  int late;                // 1: independent of the launch before it
   int* err;                // device status word (0 = ok)
   uint64_t wait_ns;        // budget of every barrier wait (the plan's)
 };
@@ -153,6 +155,10 @@ k_joint_fwd_tc(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
   }
   __syncthreads();
   tc_fence_after();
+  // a launch that follows another form of the same stage is independent of it: it starts on the
+  // SMs the first one leaves and waits for it only at its end
+  if (!args.late) pdl_wait();
+  pdl_trigger();
   const uint32_t tbase = tmem_base;
   const uint32_t t_re = tbase, t_im = tbase + BN, t_pool = tbase + 2 * BN;
 
@@ -413,6 +419,7 @@ k_joint_fwd_tc(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
     tc_fence_after();
     tmem_dealloc(tbase, 512);
   }
+  if (args.late) pdl_wait();
 }
 
 // ------------------------------------------------------------------ 16-frame form
@@ -505,6 +512,10 @@ k_joint_fwd_tc16(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
   }
   __syncthreads();
   tc_fence_after();
+  // a launch that follows another form of the same stage is independent of it: it starts on the
+  // SMs the first one leaves and waits for it only at its end
+  if (!args.late) pdl_wait();
+  pdl_trigger();
   const uint32_t tbase = tmem_base;
 
   auto fail = [&](int code) {
@@ -821,6 +832,7 @@ k_joint_fwd_tc16(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
     tc_fence_after();
     tmem_dealloc(tbase, 512);
   }
+  if (args.late) pdl_wait();
 }
 
 // ------------------------------------------------------------------ spin-pair form
@@ -906,6 +918,10 @@ k_joint_fwd_tp(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
   }
   __syncthreads();
   tc_fence_after();
+  // a launch that follows another form of the same stage is independent of it: it starts on the
+  // SMs the first one leaves and waits for it only at its end
+  if (!args.late) pdl_wait();
+  pdl_trigger();
   const uint32_t tbase = tmem_base;
   const uint32_t t_pool = tbase + 256;                   // [spin] NP columns each
   const uint32_t t_z = t_pool + 2 * NP;                  // [spin][plane] 32 columns of |Z|
@@ -1250,6 +1266,7 @@ k_joint_fwd_tp(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
     tc_fence_after();
     tmem_dealloc(tbase, 512);
   }
+  if (args.late) pdl_wait();
 }
 
 // phi_F pooling along lambda of the time-pooled rows: S2[b, a, c, lo, t] =
@@ -1262,6 +1279,7 @@ constexpr int kPoolRowsMax = 8192;   // n1 * n_t floats staged per channel
 
 __global__ void __launch_bounds__(kPoolThreads)
 k_pool_lambda(DevPlan Pd, const float* __restrict__ P, float* __restrict__ s2) {
+  pdl_enter();
   __shared__ float rows[kPoolRowsMax];
   __shared__ float phi[1024];
   const int a = blockIdx.x, b = blockIdx.y;
@@ -1737,7 +1755,8 @@ jtfs_status launch_joint_fwd_tc(const jtfs_plan* p, int B, const void* yhi_v, co
                                               cudaFuncAttributeMaxDynamicSharedMemorySize,      \
                                               (int)smem), "attr tc")) != JTFS_OK)               \
       return rc;                                                                                \
-    k_joint_fwd_tc<NTV, BNV, RESV><<<grid, kThreads, smem, st>>>(maps, args, d); ++p->prof.launches; \
+    launch_pdl(k_joint_fwd_tc<NTV, BNV, RESV>, grid, kThreads, smem, st, maps, args, d);      \
+    ++p->prof.launches;                                                                         \
   } while (0)
 #define JTFS_LAUNCH_TC16(RESV, TFV)                                                             \
   do {                                                                                          \
@@ -1745,7 +1764,8 @@ jtfs_status launch_joint_fwd_tc(const jtfs_plan* p, int B, const void* yhi_v, co
                                               cudaFuncAttributeMaxDynamicSharedMemorySize,      \
                                               (int)smem), "attr tc16")) != JTFS_OK)             \
       return rc;                                                                                \
-    k_joint_fwd_tc16<RESV, TFV><<<grid, kThreads, smem, st>>>(maps, args, d); ++p->prof.launches; \
+    launch_pdl(k_joint_fwd_tc16<RESV, TFV>, grid, kThreads, smem, st, maps, args, d);         \
+    ++p->prof.launches;                                                                         \
   } while (0)
 #define JTFS_LAUNCH_TP1(RESV, PSV, NTV)                                                         \
   do {                                                                                          \
@@ -1753,7 +1773,7 @@ jtfs_status launch_joint_fwd_tc(const jtfs_plan* p, int B, const void* yhi_v, co
                                               cudaFuncAttributeMaxDynamicSharedMemorySize,      \
                                               (int)smem), "attr tp")) != JTFS_OK)               \
       return rc;                                                                                \
-    k_joint_fwd_tp<RESV, PSV, NTV><<<grid, kTpThreads, smem, st>>>(maps, args, d);              \
+    launch_pdl(k_joint_fwd_tp<RESV, PSV, NTV>, grid, kTpThreads, smem, st, maps, args, d);      \
     ++p->prof.launches;                                                                         \
   } while (0)
 #define JTFS_LAUNCH_PAIR(RESV, PSV)                                                             \
@@ -1764,6 +1784,7 @@ jtfs_status launch_joint_fwd_tc(const jtfs_plan* p, int B, const void* yhi_v, co
     const bool res = pass == 0;
     const int first = res ? 0 : n_res, count = res ? n_res : n_all - n_res;
     if (count <= 0) continue;
+    args.late = pass == 1 && n_res > 0;
     args.items = reinterpret_cast<const int4*>(p->d_tc_items) + first;
     args.n_base = count;
     args.n_items = count * B;
@@ -1790,7 +1811,7 @@ jtfs_status launch_joint_fwd_tc(const jtfs_plan* p, int B, const void* yhi_v, co
 #undef JTFS_LAUNCH_TC16
 #undef JTFS_LAUNCH_PAIR
 #undef JTFS_LAUNCH_TP1
-  k_pool_lambda<<<dim3(p->n2, B), kPoolThreads, 0, st>>>(d, Pbuf, s2);
+  launch_pdl(k_pool_lambda, dim3(p->n2, B), kPoolThreads, 0, st, d, Pbuf, s2);
   ++p->prof.launches;
   return cuda_check(cudaGetLastError(), "k_pool_lambda");
 }

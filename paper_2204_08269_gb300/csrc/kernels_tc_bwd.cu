@@ -20,6 +20,7 @@
 #include <vector>
 
 #include "internal.h"
+#include "pdl.cuh"
 #include "tma_host.h"
 #include "umma.cuh"
 
@@ -51,6 +52,7 @@ struct TbArgs {
   int g1_rows;          // rows per (b, alpha) block of G1 = n_chunks * 32
   const int* wt_row0;   // [n2] first row of each rate in the weight table
   float2* gy;           // [B][y_len] complex FP32, rows (lambda' - lam_min) x L_alpha
+  int late;             // 1: independent of the launch before it
   int* err;
   uint64_t wait_ns;     // budget of every barrier wait (the plan's)
 };
@@ -111,6 +113,8 @@ k_joint_bwd_tc(const __grid_constant__ TbMaps maps, TbArgs args, DevPlan P) {
   }
   __syncthreads();
   tc_fence_after();
+  if (!args.late) pdl_wait();   // (a later form of the stage waits for the earlier one at its end)
+  pdl_trigger();
   const uint32_t tbase = tmem_base;
   auto fail = [&](int code) {
     if (!abort_flag) {
@@ -367,6 +371,7 @@ k_joint_bwd_tc(const __grid_constant__ TbMaps maps, TbArgs args, DevPlan P) {
     tc_fence_after();
     tmem_dealloc(tbase, 512);
   }
+  if (args.late) pdl_wait();
 }
 
 // Three-pass variant (each product split x = hi + lo: hi*hi + hi*lo + lo*hi), for FP32-level
@@ -428,6 +433,8 @@ k_joint_bwd_tc3(const __grid_constant__ Tb3Maps maps, TbArgs args, DevPlan P) {
   }
   __syncthreads();
   tc_fence_after();
+  if (!args.late) pdl_wait();   // (a later form of the stage waits for the earlier one at its end)
+  pdl_trigger();
   const uint32_t tbase = tmem_base;
   auto fail = [&](int code) {
     if (!abort_flag) {
@@ -682,6 +689,7 @@ k_joint_bwd_tc3(const __grid_constant__ Tb3Maps maps, TbArgs args, DevPlan P) {
     tc_fence_after();
     tmem_dealloc(tbase, 512);
   }
+  if (args.late) pdl_wait();
 }
 
 // ------------------------------------------------------------------ fast form
@@ -716,6 +724,7 @@ struct TfArgs {
   int a2bufs;           // gZ staging buffers (1..2)
   const int* wt_row0;
   float2* gy;
+  int late;             // 1: independent of the launch before it
   int* err;
   uint64_t wait_ns;     // budget of every barrier wait (the plan's)
 };
@@ -800,6 +809,8 @@ k_joint_bwd_fast(const __grid_constant__ TfMaps maps, TfArgs args, DevPlan P) {
   }
   __syncthreads();
   tc_fence_after();
+  if (!args.late) pdl_wait();   // (a later form of the stage waits for the earlier one at its end)
+  pdl_trigger();
   const uint32_t tbase = tmem_base;
   const uint32_t t_d2 = tbase + 6 * RC;                    // NAT x [Im 64 | Re 64]
   auto fail = [&](int code) {
@@ -1069,6 +1080,7 @@ k_joint_bwd_fast(const __grid_constant__ TfMaps maps, TfArgs args, DevPlan P) {
     tc_fence_after();
     tmem_dealloc(tbase, 512);
   }
+  if (args.late) pdl_wait();
 }
 
 // ------------------------------------------------------------------ spin-pair form
@@ -1103,6 +1115,7 @@ struct TpArgs {
   int chan_phi0;        // 2 n_fr n1: channel row of the first phi_F row
   const int* wt_row0;
   float2* gy;
+  int late;             // 1: independent of the launch before it
   int* err;
   uint64_t wait_ns;     // budget of every barrier wait (the plan's)
 };
@@ -1164,6 +1177,8 @@ k_joint_bwd_pair(const __grid_constant__ TpMaps maps, TpArgs args, DevPlan P) {
   }
   __syncthreads();
   tc_fence_after();
+  if (!args.late) pdl_wait();   // (a later form of the stage waits for the earlier one at its end)
+  pdl_trigger();
   const uint32_t tbase = tmem_base;
   // TMEM: NB1 buffers of 6 RC columns, each [P1 | P4] [P3 | P2] [g_up | g_dn] (2 RC apiece),
   // then gY^T_re and gY^T_im (64 NAT columns each), then (TA) S_re, S_im, T_re, T_im as the
@@ -1496,6 +1511,7 @@ k_joint_bwd_pair(const __grid_constant__ TpMaps maps, TpArgs args, DevPlan P) {
     tc_fence_after();
     tmem_dealloc(tbase, 512);
   }
+  if (args.late) pdl_wait();
 }
 
 // G1[(b n2 + a) g1_rows + c n1 + lambda][t] = sum_lo phi_F[(lo s_F - lambda) mod N_fr] gS2[b,a,c,lo,t]
@@ -1509,6 +1525,7 @@ constexpr int kG1InMax = 4096;       // n_lo * n_t floats of one channel
 __global__ void __launch_bounds__(kG1Threads)
 k_g1(DevPlan Pd, const float* __restrict__ gs2, int NT, int g1_rows,
      __nv_bfloat16* __restrict__ g1, __nv_bfloat16* __restrict__ g1lo) {
+  pdl_enter();
   __shared__ float gin[kG1InMax];
   __shared__ float phi[1024];
   const int a = blockIdx.x, b = blockIdx.y;
@@ -1809,7 +1826,7 @@ jtfs_status launch_joint_bwd_tc(const jtfs_plan* p, int B, const void* yhi_v, co
   __nv_bfloat16* g1hi = (__nv_bfloat16*)g1buf;
   __nv_bfloat16* g1lo = (__nv_bfloat16*)((char*)g1buf + g1_plane);
   // G1 (phi_F adjoint of g_S2), zero padded by the kernel
-  k_g1<<<dim3(p->n2, B), kG1Threads, 0, st>>>(d, gs2, NT, g1_rows, g1hi, three ? g1lo : nullptr);
+  launch_pdl(k_g1, dim3(p->n2, B), kG1Threads, 0, st, d, gs2, NT, g1_rows, g1hi, three ? g1lo : nullptr);
   ++p->prof.launches;
   if ((rc = cuda_check(cudaGetLastError(), "k_g1")) != JTFS_OK) return rc;
   std::string err;
@@ -1880,7 +1897,10 @@ jtfs_status launch_joint_bwd_tc(const jtfs_plan* p, int B, const void* yhi_v, co
   // fast form: the K1 <= 64 items (one lambda' atom, 64-row chunks), then the K1 <= KM items
   // (two atoms, 32-row chunks)
   const int n_fast = (int)(p->tcbf_items.size() / 4);
-  for (int nat = 1; nat <= 3; ++nat) {
+  // the forms write different rates and follow one another without waiting (TpArgs.late), the few
+  // items of the widest rates first: at B = 1 they take as long as all the others together
+  int launched = 0;
+  for (int nat = 3; nat >= 1; --nat) {
     const int first = nat == 1 ? 0 : (nat == 2 ? p->tcbf_n1 : n_fast - p->tcbf_n3);
     const int count = nat == 1 ? p->tcbf_n1
                                : (nat == 2 ? n_fast - p->tcbf_n1 - p->tcbf_n3 : p->tcbf_n3);
@@ -1929,7 +1949,7 @@ jtfs_status launch_joint_bwd_tc(const jtfs_plan* p, int B, const void* yhi_v, co
                                               cudaFuncAttributeMaxDynamicSharedMemorySize,      \
                                               (int)smemp), "attr tcbp")) != JTFS_OK)            \
       return rc;                                                                                \
-    k_joint_bwd_pair<PLV, NATV, KMV, RCV, NTV><<<grid, kFThreads, smemp, st>>>(pm, pa, d);     \
+    launch_pdl(k_joint_bwd_pair<PLV, NATV, KMV, RCV, NTV>, grid, kFThreads, smemp, st, pm, pa, d);\
     ++p->prof.launches;                                                                         \
   } while (0)
 #define JTFS_LAUNCH_TCBP(PLV, NATV, KMV, RCV)                                                   \
@@ -1939,7 +1959,7 @@ jtfs_status launch_joint_bwd_tc(const jtfs_plan* p, int B, const void* yhi_v, co
   } while (0)
       // one atom; two atoms with K1 <= 96 (a 96-row Y^T tile); two atoms with K1 <= 128;
       // three atoms (K1 <= 160, 16-row chunks)
-      for (int part = 0; part < (nat == 2 ? 2 : 1); ++part) {
+      for (int part = nat == 2 ? 1 : 0; part >= 0; --part) {
         const int f0 = first + (part == 1 ? p->tcbf_n2a : 0);
         const int cnt = nat != 2 ? count : (part == 0 ? p->tcbf_n2a : count - p->tcbf_n2a);
         if (cnt <= 0) continue;
@@ -1953,6 +1973,7 @@ jtfs_status launch_joint_bwd_tc(const jtfs_plan* p, int B, const void* yhi_v, co
         pa.n_items = cnt * B;
         pa.wbufs = wbp;
         pa.a2bufs = na2p;
+        pa.late = launched++ > 0;
         const int grid = std::min(pa.n_items, n_sm);
         if (three) {
           if (nat == 1) JTFS_LAUNCH_TCBP(2, 1, 64, 32);
@@ -2006,6 +2027,7 @@ jtfs_status launch_joint_bwd_tc(const jtfs_plan* p, int B, const void* yhi_v, co
     fa.g1_rows = g1_rows;
     fa.wbufs = wb;
     fa.a2bufs = na2;
+    fa.late = launched++ > 0;
     fa.wt_row0 = p->d_wtb_row0;
     fa.gy = gy;
     fa.err = p->d_err;
@@ -2017,7 +2039,8 @@ jtfs_status launch_joint_bwd_tc(const jtfs_plan* p, int B, const void* yhi_v, co
                                               cudaFuncAttributeMaxDynamicSharedMemorySize,      \
                                               (int)smem), "attr tcbf")) != JTFS_OK)             \
       return rc;                                                                                \
-    k_joint_bwd_fast<NTV, RCV, PLV, NATV, KMV><<<grid, kFThreads, smem, st>>>(fm, fa, d); ++p->prof.launches; \
+    launch_pdl(k_joint_bwd_fast<NTV, RCV, PLV, NATV, KMV>, grid, kFThreads, smem, st, fm, fa, d);\
+    ++p->prof.launches;                                                                         \
   } while (0)
 #define JTFS_LAUNCH_TCBF_NT(RCV, PLV, NATV, KMV)                                                \
   do {                                                                                          \
@@ -2039,6 +2062,7 @@ jtfs_status launch_joint_bwd_tc(const jtfs_plan* p, int B, const void* yhi_v, co
   const int PL = three ? 2 : 1;
   int n_res = three ? (NT <= 32 ? p->tcb_n_res : 0) : n_all;
   if (n_res > 0) {
+    args.late = launched++ > 0;
     args.items = reinterpret_cast<const int4*>(p->d_tcb_items);
     args.n_items = n_res * B;
     const int grid = std::min(args.n_items, n_sm);
@@ -2049,7 +2073,8 @@ jtfs_status launch_joint_bwd_tc(const jtfs_plan* p, int B, const void* yhi_v, co
                                               cudaFuncAttributeMaxDynamicSharedMemorySize,      \
                                               (int)smem), "attr tcb")) != JTFS_OK)              \
       return rc;                                                                                \
-    k_joint_bwd_tc<NTV, PLV><<<grid, kThreads, smem, st>>>(maps, args, d); ++p->prof.launches; \
+    launch_pdl(k_joint_bwd_tc<NTV, PLV>, grid, kThreads, smem, st, maps, args, d);              \
+    ++p->prof.launches;                                                                         \
   } while (0)
     if (PL == 1) {
       if (NT == 16) JTFS_LAUNCH_TCB(16, 1);
@@ -2064,6 +2089,7 @@ jtfs_status launch_joint_bwd_tc(const jtfs_plan* p, int B, const void* yhi_v, co
   }
   if (!three || n_res == n_all) return JTFS_OK;
   // streamed-Y three-pass launch for the remaining items
+  args.late = launched++ > 0;
   args.items = reinterpret_cast<const int4*>(p->d_tcb_items) + n_res;
   args.n_items = (n_all - n_res) * B;
   const int grid = std::min(args.n_items, n_sm);
@@ -2081,7 +2107,8 @@ jtfs_status launch_joint_bwd_tc(const jtfs_plan* p, int B, const void* yhi_v, co
                                               cudaFuncAttributeMaxDynamicSharedMemorySize,      \
                                               (int)smem), "attr tcb3")) != JTFS_OK)             \
       return rc;                                                                                \
-    k_joint_bwd_tc3<NTV, WBV><<<grid, kThreads, smem, st>>>(maps3, args, d); ++p->prof.launches; \
+    launch_pdl(k_joint_bwd_tc3<NTV, WBV>, grid, kThreads, smem, st, maps3, args, d);            \
+    ++p->prof.launches;                                                                         \
   } while (0)
   if (NT == 16) JTFS_LAUNCH_TCB3(16, 2);
   else if (NT == 32) JTFS_LAUNCH_TCB3(32, 2);

@@ -6,6 +6,7 @@
 
 #include "fft.cuh"
 #include "internal.h"
+#include "pdl.cuh"
 
 namespace jtfs {
 namespace {
@@ -19,6 +20,7 @@ constexpr int kRowLaunch = 256;
 // then x-hat[k] = sum_r exp(-2 pi i r k / N) X_r[k mod M].
 __global__ void __launch_bounds__(kFftThreads)
 k_xfft_sub(DevPlan P, const float* __restrict__ x, float2* __restrict__ xsub) {
+  pdl_enter();
   extern __shared__ float2 sm[];
   const int r = blockIdx.x, b = blockIdx.y;
   const float* xb = x + (size_t)b * P.N;
@@ -31,6 +33,7 @@ k_xfft_sub(DevPlan P, const float* __restrict__ x, float2* __restrict__ xsub) {
 }
 
 __global__ void k_xfft_combine(DevPlan P, const float2* __restrict__ xsub, float2* __restrict__ xh) {
+  pdl_enter();
   const int b = blockIdx.y;
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   const int half = P.N >> 1;
@@ -164,6 +167,7 @@ __global__ void __launch_bounds__(kRowBound)
 k_second_order_rows(DevPlan P, const int4* __restrict__ items, const float2* __restrict__ uh,
                     float2* __restrict__ y, __nv_bfloat16* __restrict__ yhi,
                     __nv_bfloat16* __restrict__ ylo, int B) {
+  pdl_enter();
   extern __shared__ float2 sm[];
   __shared__ int s_off[kMaxRowsPerItem], s_kend[kMaxRowsPerItem];
   __shared__ float s_inv[kMaxRowsPerItem];
