@@ -1092,9 +1092,15 @@ k_joint_bwd_fast(const __grid_constant__ TfMaps maps, TfArgs args, DevPlan P) {
 // gZ_up = a + ib and gZ_dn = c + id, W_up^H gZ_up + W_dn^H gZ_dn = Wr^T S + Wi^T T for
 // S = (a + c) + i (b + d) and T = (b - d) + i (c - a), so the last product takes four MMAs:
 //   gY^T_re += S_re Wr + T_re Wi,   gY^T_im += S_im Wr + T_im Wi   (N = 64 lambda').
-// W bytes per channel row are a third of the channel-row form's [-Wi][Wr][Wi] blocks, which
-// leaves room for a four-chunk W ring.  PL = 2: the FP32-grade split as in the fast form.
+// W bytes per channel row are a third of the channel-row form's [-Wi][Wr][Wi] blocks.
+// PL = 2: the FP32-grade split as in the fast form.
 // NT = 16 or 32 pooled frames (the K of the g product; rows of NT BF16 = 32 or 64 bytes).
+// S and T are staged in tensor memory as the last product's A operand.  One atom (NAT = 1) also
+// keeps Y^T there, the first product's A operand: it is read by every chunk of an item, and from
+// shared memory those reads (4 KB per MMA against 2 KB of W) and the S / T staging filled the
+// shared-memory pipe.  The epilogue warps copy the next item's Y^T before they write this item's
+// gY, so the copy hides behind the last chunk.  B = 64, N = 2^16, FP32-grade: contraction backward
+// 7.27 -> 6.95 ms; with S / T alone in tensor memory 7.28; with the copy after the gY write 7.06.
 struct TpMaps {
   CUtensorMap w[4];      // pair planes Wr_hi, Wi_hi, Wr_lo, Wi_lo; box {64 lambda', RC rows}
   CUtensorMap y[2][16];  // [hi/lo][alpha]: Y planes [2B][K][L], box {64 n, 32 lambda', 1}
@@ -1108,8 +1114,7 @@ struct TpArgs {
   int n_items;
   int n_chunks;         // ceil(n_pr / 32)
   int g1_rows;          // rows per (b, alpha) block of G1
-  int wbufs;            // W chunk ring depth (2..4)
-  int a2bufs;           // S / T staging buffers (1..2)
+  int wbufs;            // W chunk ring depth (2..kPairWBufs)
   int pr_phi0;          // first phi_F pair row (multiple of 32)
   int spin_rows;        // n_fr n1: channel row of the first spin-down row
   int chan_phi0;        // 2 n_fr n1: channel row of the first phi_F row
@@ -1119,6 +1124,8 @@ struct TpArgs {
   int* err;
   uint64_t wait_ns;     // budget of every barrier wait (the plan's)
 };
+
+constexpr int kPairWBufs = 6;
 
 template <int PL, int NAT, int KMV, int RCV, int NT>
 __global__ void __launch_bounds__(kFThreads, 1)
@@ -1131,40 +1138,42 @@ k_joint_bwd_pair(const __grid_constant__ TpMaps maps, TpArgs args, DevPlan P) {
   constexpr uint32_t kSw = NT * 2;                        // bytes per row of the NT-wide tiles
   constexpr uint32_t kLayNT = kSw == 64 ? kSw64 : kSw32;
   constexpr int D1C = 6 * RC;                             // first-product columns per buffer
-  constexpr int NB1 = NAT == 1 ? 2 : 1;                   // first-product TMEM buffers
-  constexpr bool TA = NAT >= 2;                           // S / T staged in TMEM (A operand)
+  constexpr bool YT = NAT == 1;                           // Y^T held in TMEM (first A operand)
+  constexpr int NA4 = YT ? 2 : 1;                         // weight tile buffers
   constexpr uint32_t kA1Plane = 2 * KM * 128;             // two 64-sample halves x 64 lambda'
   constexpr uint32_t kA4Plane = 128 * NT * 2;             // [128 n][NT t], NT * 2-byte swizzle
   constexpr uint32_t kWBlk = RC * 128;                    // RC rows x 64 lambda'
   constexpr uint32_t kG1Blk = RC * NT * 2;                // RC rows x NT t
   constexpr uint32_t kWBuf = PL * NAT * 2 * kWBlk + PL * 2 * kG1Blk;   // [Wr a][Wi a] per atom a
-  constexpr uint32_t kA2Part = 128 * RC * 2;              // [128 n][RC r] bf16, 64-byte swizzle
-  constexpr uint32_t kA2Buf = 4 * kA2Part;                // S_re, S_im, T_re, T_im
-  const int WB = args.wbufs, NA2 = args.a2bufs;
+  const int WB = args.wbufs;
   uint8_t* sA1 = sm;                                       // PL x 2 parts
-  uint8_t* sA4 = sA1 + PL * 2 * kA1Plane;                  // PL planes
-  uint8_t* sW = sA4 + PL * kA4Plane;                       // WB buffers: W blocks, then G1
-  uint8_t* sA2 = sW + WB * kWBuf;                          // NA2 buffers (shared-memory staging)
+  uint8_t* sA4 = sA1 + PL * 2 * kA1Plane;                  // NA4 buffers of PL planes
+  uint8_t* sW = sA4 + NA4 * PL * kA4Plane;                 // WB buffers: W blocks, then G1
 
-  __shared__ uint64_t a1_full, a1_free, w_full[4], w_empty[4], d1_full[2], d1_free[2],
-      a2_full[2], a2_free[2], d2_full, d2_free, mma_done, mma_done2;
+  // a1: the Y^T tile (with the weights when it stays in shared memory); a4: the weight tiles
+  // and yt: Y^T in TMEM (YT)
+  __shared__ uint64_t a1_full, a1_free, a4_full[2], a4_free[2], yt_full, w_full[kPairWBufs],
+      w_empty[kPairWBufs], d1_full, d1_free, a2_full, a2_free, d2_full, d2_free, mma_done, mma_done2;
   __shared__ uint32_t tmem_base;
   __shared__ volatile int abort_flag;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     abort_flag = 0;
     mbar_init(&a1_full, 1);
-    mbar_init(&a1_free, 1);
-    for (int i = 0; i < 4; ++i) {
+    mbar_init(&a1_free, YT ? 16 : 1);
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&a4_full[i], 1);
+      mbar_init(&a4_free[i], 1);
+    }
+    mbar_init(&yt_full, 16);
+    for (int i = 0; i < kPairWBufs; ++i) {
       mbar_init(&w_full[i], 1);
       mbar_init(&w_empty[i], 1);
     }
-    for (int i = 0; i < 2; ++i) {
-      mbar_init(&d1_full[i], 1);
-      mbar_init(&d1_free[i], 16);
-      mbar_init(&a2_full[i], 16);
-      mbar_init(&a2_free[i], 1);
-    }
+    mbar_init(&d1_full, 1);
+    mbar_init(&d1_free, 16);
+    mbar_init(&a2_full, 16);
+    mbar_init(&a2_free, 1);
     mbar_init(&d2_full, 1);
     mbar_init(&d2_free, 16);
     mbar_init(&mma_done, 1);
@@ -1180,12 +1189,13 @@ k_joint_bwd_pair(const __grid_constant__ TpMaps maps, TpArgs args, DevPlan P) {
   if (!args.late) pdl_wait();   // (a later form of the stage waits for the earlier one at its end)
   pdl_trigger();
   const uint32_t tbase = tmem_base;
-  // TMEM: NB1 buffers of 6 RC columns, each [P1 | P4] [P3 | P2] [g_up | g_dn] (2 RC apiece),
-  // then gY^T_re and gY^T_im (64 NAT columns each), then (TA) S_re, S_im, T_re, T_im as the
-  // last product's A operand: RC pair rows of BF16 = RC / 2 columns apiece
-  static_assert(NB1 * D1C + 128 * NAT + (TA ? 2 * RC : 0) <= 512, "TMEM columns");
-  const uint32_t t_re = tbase + NB1 * D1C, t_im = t_re + 64 * NAT;
-  const uint32_t t_a2 = t_im + 64 * NAT;
+  // TMEM: 6 RC columns [P1 | P4] [P3 | P2] [g_up | g_dn] (2 RC apiece), then gY^T_re and gY^T_im
+  // (64 NAT columns each), then S_re, S_im, T_re, T_im as the last product's A operand (RC pair
+  // rows of BF16 = RC / 2 columns apiece), then (YT) the planes Yr_hi, Yi_hi, Yr_lo, Yi_lo as the
+  // first product's (64 lambda' of BF16 = 32 columns apiece)
+  static_assert(D1C + 128 * NAT + 2 * RC + (YT ? PL * 64 : 0) <= 512, "TMEM columns");
+  const uint32_t t_re = tbase + D1C, t_im = t_re + 64 * NAT;
+  const uint32_t t_a2 = t_im + 64 * NAT, t_y = t_a2 + 2 * RC;
   auto fail = [&](int code) {
     if (!abort_flag) {
       abort_flag = 1;
@@ -1200,7 +1210,8 @@ k_joint_bwd_pair(const __grid_constant__ TpMaps maps, TpArgs args, DevPlan P) {
       uint32_t a1_ph = 0, wph = 0;
       int wst = 0;
       uint32_t armed_w = 0, armed_w_par = 0;
-      int armed_a1 = -1;
+      int armed_a1 = -1, armed_a4[2] = {-1, -1}, a4b = 0;
+      uint32_t a4_ph = 0;
       bool ok = true;
       for (int it = blockIdx.x; it < args.n_items && ok && !abort_flag; it += gridDim.x) {
         const int4 item = args.items[it % args.n_base];
@@ -1208,18 +1219,29 @@ k_joint_bwd_pair(const __grid_constant__ TpMaps maps, TpArgs args, DevPlan P) {
         const Rate2 A = P.rates2[a];
         const int nkb1 = (K1 + 31) / 32;
         if (!mbar_wait(&a1_free, a1_ph ^ 1, wait_budget)) { fail(81); break; }
-        mbar_arrive_expect_tx(&a1_full, PL * 2 * 2 * nkb1 * 4096 + PL * kA4Plane);
+        mbar_arrive_expect_tx(&a1_full, PL * 2 * 2 * nkb1 * 4096 + (YT ? 0 : PL * kA4Plane));
         armed_a1 = (int)a1_ph;
-        for (int pl = 0; pl < PL; ++pl) {
+        for (int pl = 0; pl < PL; ++pl)
           for (int part = 0; part < 2; ++part)
             for (int h = 0; h < 2; ++h)
               for (int kb = 0; kb < nkb1; ++kb)
                 tma_load_3d(sA1 + (pl * 2 + part) * kA1Plane + h * KM * 128 + kb * 32 * 128,
                             &maps.y[pl][a], n0 + h * 64, start - A.lam_min + kb * 32,
                             2 * b + part, &a1_full);
-          tma_load_2d(sA4 + pl * kA4Plane, &maps.wt[pl], 0, args.wt_row0[a] + n0, &a1_full);
-        }
         a1_ph ^= 1;
+        uint64_t* a4_bar = &a1_full;
+        if (YT) {
+          if (!mbar_wait(&a4_free[a4b], a4_ph ^ 1, wait_budget)) { fail(92); break; }
+          a4_bar = &a4_full[a4b];
+          mbar_arrive_expect_tx(a4_bar, PL * kA4Plane);
+          armed_a4[a4b] = (int)a4_ph;
+        }
+        for (int pl = 0; pl < PL; ++pl)
+          tma_load_2d(sA4 + (a4b * PL + pl) * kA4Plane, &maps.wt[pl], 0, args.wt_row0[a] + n0, a4_bar);
+        if (YT) {
+          a4_ph ^= (uint32_t)a4b;
+          a4b ^= 1;
+        }
         const int g1row = (b * P.n2 + a) * args.g1_rows;
         for (int j = 0; j < args.n_chunks; ++j) {
           if (!mbar_wait(&w_empty[wst], wph ^ 1, wait_budget)) { fail(82); ok = false; break; }
@@ -1248,29 +1270,31 @@ k_joint_bwd_pair(const __grid_constant__ TpMaps maps, TpArgs args, DevPlan P) {
       for (int i = 0; i < WB; ++i)
         if (armed_w >> i & 1) mbar_wait(&w_full[i], armed_w_par >> i & 1, wait_budget);
       if (armed_a1 >= 0) mbar_wait(&a1_full, (uint32_t)armed_a1, wait_budget);
+      for (int i = 0; i < 2; ++i)
+        if (armed_a4[i] >= 0) mbar_wait(&a4_full[i], (uint32_t)armed_a4[i], wait_budget);
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ first-product issuer
     if (elect_one()) {
-      const uint32_t id1 = instr_desc(128, 2 * RC, 1, 1, 1, 0, 0);
+      const uint32_t id1 = instr_desc(128, 2 * RC, 1, 1, YT ? 0 : 1, 0, 0);
       const uint32_t id4 = instr_desc(128, 2 * RC, 1, 1, 0, 0, 0);
-      uint32_t a1_ph = 0, wph = 0;
-      uint32_t d1f_ph = 0;   // bit i: phase of buffer i
-      int wst = 0, buf = 0;
+      uint32_t a1_ph = 0, a4_ph = 0, wph = 0, d1f_ph = 0;
+      int wst = 0, a4b = 0;
       bool ok = true;
       for (int it = blockIdx.x; it < args.n_items && ok && !abort_flag; it += gridDim.x) {
         const int4 item = args.items[it % args.n_base];
         const int nks1 = item.w / 16;
-        if (!mbar_wait(&a1_full, a1_ph, wait_budget)) { fail(83); break; }
+        if (!mbar_wait(YT ? &yt_full : &a1_full, a1_ph, wait_budget)) { fail(83); break; }
         a1_ph ^= 1;
-        const uint32_t a1 = smem_u32(sA1), a4 = smem_u32(sA4);
+        if (YT && !mbar_wait(&a4_full[a4b], a4_ph, wait_budget)) { fail(93); break; }
+        const uint32_t a1 = smem_u32(sA1), a4 = smem_u32(sA4 + a4b * PL * kA4Plane);
         for (int j = 0; j < args.n_chunks && ok; ++j) {
           if (!mbar_wait(&w_full[wst], wph, wait_budget)) { fail(84); ok = false; break; }
-          if (!mbar_wait(&d1_free[buf], ((d1f_ph >> buf) & 1) ^ 1, wait_budget)) { fail(85); ok = false; break; }
-          d1f_ph ^= 1u << buf;
+          if (!mbar_wait(&d1_free, d1f_ph ^ 1, wait_budget)) { fail(85); ok = false; break; }
+          d1f_ph ^= 1;
           tc_fence_after();
           const uint32_t wb = smem_u32(sW + wst * kWBuf);
-          const uint32_t t_a = tbase + buf * D1C, t_b = t_a + 2 * RC, t_g = t_a + 4 * RC;
+          const uint32_t t_a = tbase, t_b = t_a + 2 * RC, t_g = t_a + 4 * RC;
           // descriptors from two bases plus constant offsets (16-byte units)
           const uint64_t dY = smem_desc(a1, KM * 128, 1024, kSw128);
           const uint64_t dW = smem_desc(wb, 16, 1024, kSw128);
@@ -1286,8 +1310,13 @@ k_joint_bwd_pair(const __grid_constant__ TpMaps maps, TpArgs args, DevPlan P) {
                   const uint64_t bw =
                       dW + (uint64_t)((((pb * NAT + (ks >> 2)) * 2) * kWBlk + (ks & 3) * 32) >> 4);
                   const uint32_t f = (ks | q) ? 1u : 0u;
-                  mma_f16(t_a, ayr, bw, id1, f);    // [P1 | P4] = Yr [Wr ; Wi]^T
-                  mma_f16(t_b, ayi, bw, id1, f);    // [P3 | P2] = Yi [Wr ; Wi]^T
+                  if (YT) {
+                    mma_f16_ta(t_a, t_y + pa * 64 + ks * 8, bw, id1, f);        // Yr [Wr ; Wi]^T
+                    mma_f16_ta(t_b, t_y + pa * 64 + 32 + ks * 8, bw, id1, f);   // Yi [Wr ; Wi]^T
+                  } else {
+                    mma_f16(t_a, ayr, bw, id1, f);    // [P1 | P4] = Yr [Wr ; Wi]^T
+                    mma_f16(t_b, ayi, bw, id1, f);    // [P3 | P2] = Yi [Wr ; Wi]^T
+                  }
                 }
               }
             }
@@ -1301,12 +1330,15 @@ k_joint_bwd_pair(const __grid_constant__ TpMaps maps, TpArgs args, DevPlan P) {
                       smem_desc(g1 + pb * 2 * kG1Blk + ks * 32, 16, 8 * kSw, kLayNT), id4,
                       (q | ks) ? 1u : 0u);
           }
-          mma_commit(&d1_full[buf]);
+          mma_commit(&d1_full);
           if (++wst == WB) { wst = 0; wph ^= 1; }
-          if (NB1 == 2) buf ^= 1;
         }
         if (!ok) break;
-        mma_commit(&a1_free);
+        mma_commit(YT ? &a4_free[a4b] : &a1_free);
+        if (YT) {
+          a4_ph ^= (uint32_t)a4b;
+          a4b ^= 1;
+        }
       }
       mma_commit(&mma_done);
       mbar_wait(&mma_done, 0, wait_budget);
@@ -1315,13 +1347,13 @@ k_joint_bwd_pair(const __grid_constant__ TpMaps maps, TpArgs args, DevPlan P) {
     // ------------------------------------------------------------ last-product issuer
     if (elect_one()) {
       const uint32_t id2 = instr_desc(128, 64 * NAT, 1, 1, 0, 1, 0);
-      uint32_t d2f_ph = 0, wph = 0, a2_ph = 0;   // a2_ph bit i: phase of buffer i
-      int wst = 0, q2 = 0;
+      uint32_t d2f_ph = 0, wph = 0, a2_ph = 0;
+      int wst = 0;
       bool ok = true;
       for (int it = blockIdx.x; it < args.n_items && ok && !abort_flag; it += gridDim.x) {
         for (int j = 0; j < args.n_chunks && ok; ++j) {
-          if (!mbar_wait(&a2_full[q2], (a2_ph >> q2) & 1, wait_budget)) { fail(86); ok = false; break; }
-          a2_ph ^= 1u << q2;
+          if (!mbar_wait(&a2_full, a2_ph, wait_budget)) { fail(86); ok = false; break; }
+          a2_ph ^= 1;
           if (!mbar_wait(&w_full[wst], wph, wait_budget)) { fail(87); ok = false; break; }
           if (j == 0) {
             if (!mbar_wait(&d2_free, d2f_ph ^ 1, wait_budget)) { fail(88); ok = false; break; }
@@ -1329,41 +1361,27 @@ k_joint_bwd_pair(const __grid_constant__ TpMaps maps, TpArgs args, DevPlan P) {
           }
           tc_fence_after();
           const uint32_t wb = smem_u32(sW + wst * kWBuf);
-          const uint32_t a2 = smem_u32(sA2 + q2 * kA2Buf);
-          // descriptors from two bases plus constant offsets (16-byte units)
-          const uint64_t dS = smem_desc(a2, 16, 512, kSw64);
+          // descriptors from one base plus constant offsets (16-byte units)
           // MN-major over lambda': the NAT atoms of Wr (of Wi) are 2 kWBlk apart
           const uint64_t dW = smem_desc(wb, 2 * kWBlk, 1024, kSw128);
 #pragma unroll
           for (int ks = 0; ks < RC / 16; ++ks) {
-            const uint64_t sre = dS + (uint64_t)((0 * kA2Part + ks * 32) >> 4);
-            const uint64_t sim = dS + (uint64_t)((1 * kA2Part + ks * 32) >> 4);
-            const uint64_t tre = dS + (uint64_t)((2 * kA2Part + ks * 32) >> 4);
-            const uint64_t tim = dS + (uint64_t)((3 * kA2Part + ks * 32) >> 4);
 #pragma unroll
             for (int q = 0; q < PL; ++q) {                      // W_hi, then W_lo
               const uint32_t wo = q * NAT * 2 * kWBlk + ks * 2048;
               const uint64_t wr = dW + (uint64_t)(wo >> 4);
               const uint64_t wi = dW + (uint64_t)((wo + kWBlk) >> 4);
               const uint32_t f = (j == 0 && ks == 0 && q == 0) ? 0u : 1u;
-              if (TA) {
-                const uint32_t ta = t_a2 + ks * 8;
-                mma_f16_ta(t_re, ta, wr, id2, f);
-                mma_f16_ta(t_re, ta + RC, wi, id2, 1u);
-                mma_f16_ta(t_im, ta + RC / 2, wr, id2, f);
-                mma_f16_ta(t_im, ta + 3 * RC / 2, wi, id2, 1u);
-              } else {
-                mma_f16(t_re, sre, wr, id2, f);
-                mma_f16(t_re, tre, wi, id2, 1u);
-                mma_f16(t_im, sim, wr, id2, f);
-                mma_f16(t_im, tim, wi, id2, 1u);
-              }
+              const uint32_t ta = t_a2 + ks * 8;
+              mma_f16_ta(t_re, ta, wr, id2, f);
+              mma_f16_ta(t_re, ta + RC, wi, id2, 1u);
+              mma_f16_ta(t_im, ta + RC / 2, wr, id2, f);
+              mma_f16_ta(t_im, ta + 3 * RC / 2, wi, id2, 1u);
             }
           }
-          mma_commit(&a2_free[q2]);
+          mma_commit(&a2_free);
           mma_commit(&w_empty[wst]);
           if (++wst == WB) { wst = 0; wph ^= 1; }
-          if (++q2 == NA2) q2 = 0;
         }
         if (!ok) break;
         mma_commit(&d2_full);
@@ -1378,19 +1396,52 @@ k_joint_bwd_pair(const __grid_constant__ TpMaps maps, TpArgs args, DevPlan P) {
     const int cg = ew >> 2;                    // pair rows [8 cg, 8 cg + 8) of a chunk
     const int row = quarter * 32 + lane;       // time sample within the tile
     const uint32_t lane_off = (uint32_t)(quarter * 32) << 16;
-    uint32_t d2_ph = 0;
-    uint32_t d1_ph = 0, a2f_ph = 0;   // bit i: phase of buffer i
-    int buf = 0, q2 = 0;
+    uint32_t d2_ph = 0, d1_ph = 0, a2f_ph = 0, y_ph = 0;
+    // YT: this warp's 32 samples of plane cg of an item's Y^T tile (shared memory, [lambda'][64
+    // samples] rows of 128 swizzled bytes) into TMEM, sample n in lane n, two lambda' per column.
+    // The caller has seen the last first product of the item before complete.
+    auto stage_y = [&](int nks1) -> bool {
+      if (!mbar_wait(&a1_full, y_ph, wait_budget)) { fail(94); return false; }
+      y_ph ^= 1;
+      tc_fence_after();
+      if (cg < 2 * PL) {
+        const int n = row & 63;
+        const uint8_t* y = sA1 + cg * kA1Plane + (row >> 6) * KM * 128 + (n & 7) * 2;
+        for (int ks = 0; ks < nks1; ++ks) {
+          uint32_t v[8];
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            const int l0 = 2 * i, l1 = 2 * i + 1;   // lambda' within the 16
+            const uint32_t e0 = *reinterpret_cast<const uint16_t*>(
+                y + (ks * 16 + l0) * 128 + (((n >> 3) ^ (l0 & 7)) << 4));
+            const uint32_t e1 = *reinterpret_cast<const uint16_t*>(
+                y + (ks * 16 + l1) * 128 + (((n >> 3) ^ (l1 & 7)) << 4));
+            v[i] = e0 | (e1 << 16);
+          }
+          tmem_st8(t_y + lane_off + cg * 32 + ks * 8, v);
+        }
+      }
+      tmem_wait_st();
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) {
+        mbar_arrive(&a1_free);
+        mbar_arrive(&yt_full);
+      }
+      return true;
+    };
+    bool staged = true;
+    if (YT && (int)blockIdx.x < args.n_items) staged = stage_y(args.items[blockIdx.x % args.n_base].w / 16);
     for (int it = blockIdx.x; it < args.n_items; it += gridDim.x) {
       const int4 item = args.items[it % args.n_base];
       const int a = item.x, b = it / args.n_base, n0 = item.y, start = item.z;
-      bool ok = !abort_flag;
+      bool ok = !abort_flag && staged;
       for (int j = 0; j < args.n_chunks && ok; ++j) {
-        if (!mbar_wait(&d1_full[buf], (d1_ph >> buf) & 1, wait_budget)) { fail(89); ok = false; break; }
-        d1_ph ^= 1u << buf;
+        if (!mbar_wait(&d1_full, d1_ph, wait_budget)) { fail(89); ok = false; break; }
+        d1_ph ^= 1;
         tc_fence_after();
         uint32_t p1[CW], p4[CW], p3[CW], p2[CW], gu[CW], gd[CW];
-        const uint32_t t = tbase + buf * D1C + lane_off + cg * CW;
+        const uint32_t t = tbase + lane_off + cg * CW;
         if constexpr (CW == 8) {
           tmem_ld8u(t, p1);
           tmem_ld8u(t + RC, p4);
@@ -1409,7 +1460,7 @@ k_joint_bwd_pair(const __grid_constant__ TpMaps maps, TpArgs args, DevPlan P) {
         tmem_wait_ld();
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(&d1_free[buf]);
+        if (lane == 0) mbar_arrive(&d1_free);
         // phi_F rows have no spin-down channel: their g_dn copy is dropped
         if (j * RC >= args.pr_phi0) {
 #pragma unroll
@@ -1445,9 +1496,9 @@ k_joint_bwd_pair(const __grid_constant__ TpMaps maps, TpArgs args, DevPlan P) {
           tre[i] = *reinterpret_cast<uint32_t*>(&h2);
           tim[i] = *reinterpret_cast<uint32_t*>(&h3);
         }
-        if (!mbar_wait(&a2_free[q2], ((a2f_ph >> q2) & 1) ^ 1, wait_budget)) { fail(90); ok = false; break; }
-        a2f_ph ^= 1u << q2;
-        if (TA) {
+        if (!mbar_wait(&a2_free, a2f_ph ^ 1, wait_budget)) { fail(90); ok = false; break; }
+        a2f_ph ^= 1;
+        {
           // this warp's CW pair rows are columns [cg CW / 2, +CW / 2) of each part
           const uint32_t ta = t_a2 + lane_off + cg * (CW / 2);
           tc_fence_after();
@@ -1464,21 +1515,14 @@ k_joint_bwd_pair(const __grid_constant__ TpMaps maps, TpArgs args, DevPlan P) {
           }
           tmem_wait_st();
           tc_fence_before();
-        } else if constexpr (CW == 8) {
-          uint8_t* base = sA2 + q2 * kA2Buf + row * (RC * 2);
-          const int pos = (cg ^ ((row >> 1) & 3)) * 16;
-          *reinterpret_cast<uint4*>(base + 0 * kA2Part + pos) = make_uint4(sre[0], sre[1], sre[2], sre[3]);
-          *reinterpret_cast<uint4*>(base + 1 * kA2Part + pos) = make_uint4(sim[0], sim[1], sim[2], sim[3]);
-          *reinterpret_cast<uint4*>(base + 2 * kA2Part + pos) = make_uint4(tre[0], tre[1], tre[2], tre[3]);
-          *reinterpret_cast<uint4*>(base + 3 * kA2Part + pos) = make_uint4(tim[0], tim[1], tim[2], tim[3]);
-          fence_proxy_async_smem();
         }
         __syncwarp();
-        if (lane == 0) mbar_arrive(&a2_full[q2]);
-        if (NB1 == 2) buf ^= 1;
-        if (++q2 == NA2) q2 = 0;
+        if (lane == 0) mbar_arrive(&a2_full);
       }
       if (!ok) break;
+      // the next item's Y^T before this item's results: its first product runs meanwhile
+      if (YT && it + (int)gridDim.x < args.n_items)
+        staged = stage_y(args.items[(it + (int)gridDim.x) % args.n_base].w / 16);
       // gY of this tile: lambda' = start + c for c in [16 cg, 16 cg + 16)
       if (!mbar_wait(&d2_full, d2_ph, wait_budget)) { fail(91); break; }
       d2_ph ^= 1;
@@ -1634,25 +1678,21 @@ static bool tcbf_layout(const jtfs_plan* p, int nat, int* wb_out, int* na2_out, 
   return true;
 }
 
-// Shared memory of the spin-pair form: resident Y^T and weight tiles, the W ring (2..4 chunks
-// of 32 pair rows) and the S / T staging (1..2 buffers), deepest first.
+// Shared memory of the spin-pair form: the Y^T tile and the weight tiles (two for one atom, whose
+// Y^T moves on to TMEM), and the deepest W ring (2 to kPairWBufs chunks) that fits beside them.
 static int tcbp_rc(int nat) { return nat >= 3 ? 16 : 32; }
 
-static bool tcbp_layout(const jtfs_plan* p, int nat, int KM, int* wb_out, int* na2_out,
-                        size_t* smem_out) {
+static bool tcbp_layout(const jtfs_plan* p, int nat, int KM, int* wb_out, size_t* smem_out) {
   const int PL = p->split ? 2 : 1, RC = tcbp_rc(nat), NT = tc_nt(p->n_t);
-  const size_t fixed = 1024 + (size_t)PL * 2 * (2 * KM * 128) + (size_t)PL * 128 * NT * 2;
+  const size_t fixed = 1024 + (size_t)PL * 2 * (2 * KM * 128) +
+                       (size_t)(nat == 1 ? 2 : 1) * PL * 128 * NT * 2;
   const size_t wbuf = (size_t)PL * nat * 2 * RC * 128 + (size_t)PL * 2 * RC * NT * 2;
-  const size_t a2buf = nat >= 2 ? 0 : (size_t)4 * 128 * RC * 2;   // two atoms and more: S / T in TMEM
   const size_t budget = 225 * 1024;
-  int wb = 4, na2 = nat >= 2 ? 1 : 2;
-  while (fixed + wb * wbuf + na2 * a2buf > budget && (wb > 2 || na2 > 1)) {
-    if (na2 > 1 && wb == 2) na2 = 1; else --wb;
-  }
-  if (fixed + wb * wbuf + na2 * a2buf > budget) return false;
+  int wb = nat == 1 ? kPairWBufs : 4;
+  while (fixed + wb * wbuf > budget && wb > 2) --wb;
+  if (fixed + wb * wbuf > budget) return false;
   *wb_out = wb;
-  *na2_out = na2;
-  *smem_out = fixed + wb * wbuf + na2 * a2buf;
+  *smem_out = fixed + wb * wbuf;
   return true;
 }
 
@@ -1693,9 +1733,9 @@ jtfs_status build_tcb_tables(jtfs_plan* p) {
   // spin-pair form (16 or 32 frames): one atom (K1 <= 64) for the FP32-grade split, two
   // (K1 <= 128) and three (K1 <= 160) atoms for every BF16-plane precision
   const bool pair = NT <= 32 && p->d_wpair[0] != nullptr;
-  const bool use_p1 = pair && p->split && tcbp_layout(p, 1, 64, &wb_, &na2_, &smem_);
-  const bool use_p2 = pair && tcbp_layout(p, 2, 128, &wb_, &na2_, &smem_);
-  const bool use_p3 = pair && tcbp_layout(p, 3, 160, &wb_, &na2_, &smem_);
+  const bool use_p1 = pair && p->split && tcbp_layout(p, 1, 64, &wb_, &smem_);
+  const bool use_p2 = pair && tcbp_layout(p, 2, 128, &wb_, &smem_);
+  const bool use_p3 = pair && tcbp_layout(p, 3, 160, &wb_, &smem_);
   const bool use_f1 = use_p1 || tcbf_layout(p, 1, &wb_, &na2_, &smem_);
   const bool use_f2 = use_p2 || tcbf_layout(p, 2, &wb_, &na2_, &smem_);
   const int km2 = use_p2 ? 128 : tcbf_km(p, 2);
@@ -1905,10 +1945,10 @@ jtfs_status launch_joint_bwd_tc(const jtfs_plan* p, int B, const void* yhi_v, co
     const int count = nat == 1 ? p->tcbf_n1
                                : (nat == 2 ? n_fast - p->tcbf_n1 - p->tcbf_n3 : p->tcbf_n3);
     if (count <= 0) continue;
-    int wbp = 0, na2p = 0;
+    int wbp = 0;
     size_t smemp = 0;
     if (NT <= 32 && (three || nat >= 2) && p->d_wpair[0] &&
-        tcbp_layout(p, nat, nat == 1 ? 64 : (nat == 2 ? 128 : 160), &wbp, &na2p, &smemp)) {
+        tcbp_layout(p, nat, nat == 1 ? 64 : (nat == 2 ? 128 : 160), &wbp, &smemp)) {
       const int RCp = tcbp_rc(nat);
       // the spin-pair form: every atom count for the FP32-grade split, two and three atoms for
       // one BF16 pass (whose one-atom items keep the channel-row form's 128-wide products)
@@ -1964,7 +2004,7 @@ jtfs_status launch_joint_bwd_tc(const jtfs_plan* p, int B, const void* yhi_v, co
         const int cnt = nat != 2 ? count : (part == 0 ? p->tcbf_n2a : count - p->tcbf_n2a);
         if (cnt <= 0) continue;
         const int KMp = nat == 1 ? 64 : (nat == 3 ? 160 : (part == 0 ? 96 : 128));
-        if (!tcbp_layout(p, nat, KMp, &wbp, &na2p, &smemp)) {
+        if (!tcbp_layout(p, nat, KMp, &wbp, &smemp)) {
           set_error("tensor-core backward: no shared-memory layout for the spin-pair form");
           return JTFS_ERR_UNSUPPORTED;
         }
@@ -1972,7 +2012,6 @@ jtfs_status launch_joint_bwd_tc(const jtfs_plan* p, int B, const void* yhi_v, co
         pa.n_base = cnt;
         pa.n_items = cnt * B;
         pa.wbufs = wbp;
-        pa.a2bufs = na2p;
         pa.late = launched++ > 0;
         const int grid = std::min(pa.n_items, n_sm);
         if (three) {
