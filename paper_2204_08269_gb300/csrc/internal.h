@@ -131,8 +131,14 @@ struct jtfs_plan {
                                // the spin-up and phi_F rows: [n_pr][n1_pad] bf16 (16 or 32 frames)
   void* d_wtf;                 // pooling weights hi / lo: [n2 * NT][tc_wt_cols] bf16
   int tc_wt_cols;
-  std::vector<int> tc_items;   // (alpha, m0, n_tiles, 0) per signal; resident-W items first
-  int tc_n_res;                // items whose W tile fits the resident form
+  std::vector<int> tc_items;   // (alpha, m0, n_tiles, first tile) per signal and level; in each
+                               // level the resident-W items first
+  struct TcLevel {             // the rates in parts of at most cap tiles
+    int first, n, n_res;       // its items in tc_items; those whose W tile fits the resident form
+    int cap, parts;            // tiles of a part, parts of the longest rate
+    long long max_cost, cost;  // of the longest item and of all items
+  };
+  std::vector<TcLevel> tc_levels;
   int* d_tc_items;
   int* d_err;                  // device status word: 0 ok, kErrNumeric after a non-finite
                                // output, any other code from a bounded wait that gave up
@@ -214,6 +220,16 @@ std::vector<int> build_rowitems(const jtfs_plan* p, int cap);
 jtfs_status autotune_rows(jtfs_plan* p, int B, const Workspace& w, cudaStream_t st,
                           int* best_threads, int* best_cap, float* best_ms);
 
+// Blocks that the C channels of one (rate, signal) are split over in the phi_F pooling and its
+// adjoint: one where the (rate, signal) pairs fill the SMs four times, else as many as do.  One
+// block that walks all 19 channels left most SMs idle for small batches (B = 1, N = 2^16, 13
+// rates: 55 us pooling, 59 us adjoint; together with the parts below the step 855 -> 646 us).
+inline int channel_split(const jtfs_plan* p, int B, int n_sm) {
+  const long long pairs = (long long)p->n2 * B;
+  const long long z = (4LL * n_sm + pairs - 1) / pairs;
+  return (int)(z < 1 ? 1 : (z > p->C ? p->C : z));
+}
+
 // tensor-core contraction (kernels_tc.cu)
 bool tc_supported(const jtfs_plan* p);
 int tc_nt(int n_t);
@@ -237,7 +253,7 @@ jtfs_status launch_scat1d_backward(const jtfs_plan* p, const float* x, const flo
                                    float* gx, const Workspace& w, cudaStream_t st);
 jtfs_status launch_wait_diagnostic(const jtfs_plan* p, uint64_t budget_ns, cudaStream_t st);
 jtfs_status launch_joint_fwd_tc(const jtfs_plan* p, int B, const void* yhi, const void* ylo,
-                                float* Pbuf, float* s2, cudaStream_t st);
+                                float* Pbuf, float* part_buf, float* s2, cudaStream_t st);
 
 bool tcb_supported(const jtfs_plan* p);
 jtfs_status build_tcb_tables(jtfs_plan* p);

@@ -584,7 +584,7 @@ jtfs_status launch_forward(const jtfs_plan* p, const float* x, int B, float* s0,
       }
     }
     StageScope sc(p, kStJointFwd, st, 0);   // the launcher counts its kernels
-    jtfs_status r2 = launch_joint_fwd_tc(p, B, w.yt, nullptr, w.pbuf, s2, st);
+    jtfs_status r2 = launch_joint_fwd_tc(p, B, w.yt, nullptr, w.pbuf, nullptr, s2, st);
     if (r2 != JTFS_OK) return r2;
   } else if (p->use_tc) {
     if (!p->pairs.empty()) {
@@ -592,7 +592,8 @@ jtfs_status launch_forward(const jtfs_plan* p, const float* x, int B, float* s0,
       launch_pdl(k_second_order_rows<1>, dim3((unsigned)(p->rowitems.size() / 4), B), p->row_threads, (size_t)p->rows_cap * 17 / 2, st, d, reinterpret_cast<const int4*>(p->d_rowitems), w.uh, nullptr, (__nv_bfloat16*)w.ybh, (__nv_bfloat16*)w.ybl, B);
     }
     StageScope sc(p, kStJointFwd, st, 0);   // the launcher counts its kernels
-    jtfs_status r2 = launch_joint_fwd_tc(p, B, w.ybh, w.ybl, w.pbuf, s2, st);
+    // (the FP32 Y buffer is free here)
+    jtfs_status r2 = launch_joint_fwd_tc(p, B, w.ybh, w.ybl, w.pbuf, reinterpret_cast<float*>(w.y), s2, st);
     if (r2 != JTFS_OK) return r2;
   } else {
     if (!p->pairs.empty()) {

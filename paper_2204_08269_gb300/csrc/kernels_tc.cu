@@ -51,9 +51,10 @@ struct TcMaps {
 };
 
 struct TcArgs {
-  const int4* items;       // (alpha, m0, n_tiles, 0) per base, longest first
+  const int4* items;       // (alpha, m0, n_tiles, first tile) per base, longest first
   int n_base;              // bases; item it = base it % n_base of signal it / n_base, so the
                            // row tiles of one signal's Y run together and share it in L2
+  int split;               // 1: rates split over parts (small batches): base it / B of signal it % B
   int n_items;             // n_base * B
   int B;
   int passes;              // 1 or 3
@@ -65,11 +66,25 @@ struct TcArgs {
   int pr_phi0;             // spin-pair form: first phi_F pair row
   int nt;                  // frames
   float* P;                // [B][n2][C*n1][nt]
+  float* P2;               // the same for the parts 1, 2, ... of split rates, part_stride apart
+  long long part_stride;
+  int part_tiles;          // tiles of one part
   int n2;
   int late;                // 1: independent of the launch before it
   int* err;                // device status word (0 = ok)
   uint64_t wait_ns;        // budget of every barrier wait (the plan's)
 };
+
+__device__ __forceinline__ int4 tc_item(const TcArgs& args, int it, int& b) {
+  const int base = args.split ? it / args.B : it % args.n_base;
+  b = args.split ? it - base * args.B : it / args.n_base;
+  return args.items[base];
+}
+// where the part that starts at this tile writes its pooled rows
+__device__ __forceinline__ float* tc_partial(const TcArgs& args, int tile0) {
+  const int q = tile0 / args.part_tiles;
+  return q ? args.P2 + (q - 1) * args.part_stride : args.P;
+}
 
 // 32 lanes x 32 bits, 32 consecutive columns per thread.
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
@@ -179,8 +194,9 @@ k_joint_fwd_tc(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
       int armed_a = -1;
       bool ok = true;
       for (int it = blockIdx.x; it < args.n_items && ok && !abort_flag; it += gridDim.x) {
-        const int4 item = args.items[it % args.n_base];
-        const int a = item.x, b = it / args.n_base, m0 = item.y, ntiles = item.z;
+        int b;
+        const int4 item = tc_item(args, it, b);
+        const int a = item.x, m0 = item.y, ntiles = item.z;
         const Rate2 A = P.rates2[a];
         const int lm8 = A.lam_min & ~7;
         const int nkb = (((P.n1 - lm8 + 15) >> 4) + 1) >> 1;
@@ -211,7 +227,7 @@ k_joint_fwd_tc(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
                               lm8 + kb * kBK, m0, &full_bar[stage]);
                 for (int h = 0; h < NH; ++h)
                   tma_load_3d(sb + ((pl * 2 + part) * NH + h) * kBHalf, &maps.y[pl][a],
-                              j * BN + h * 64, lm8 + kb * kBK - A.lam_min, 2 * b + part,
+                              (item.w + j) * BN + h * 64, lm8 + kb * kBK - A.lam_min, 2 * b + part,
                               &full_bar[stage]);
               }
             }
@@ -225,7 +241,7 @@ k_joint_fwd_tc(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
           for (int pl = 0; pl < planes; ++pl)
             for (int h = 0; h < NH; ++h)
               tma_load_2d(sWt + ((ws * planes + pl) * NH + h) * kWHalf, &maps.wt[pl],
-                          j * BN + h * 64, a * NT, &wfull[ws]);
+                          (item.w + j) * BN + h * 64, a * NT, &wfull[ws]);
           if (++ws == WS) { ws = 0; wph ^= 1; }
         }
       }
@@ -247,7 +263,8 @@ k_joint_fwd_tc(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
       uint32_t phase = 0, tph = 0, zph = 0, wph = 0, d3ph = 0, aph = 0;
       bool ok = true;
       for (int it = blockIdx.x; it < args.n_items && ok && !abort_flag; it += gridDim.x) {
-        const int4 item = args.items[it % args.n_base];
+        int b;
+        const int4 item = tc_item(args, it, b);
         const Rate2 A = P.rates2[item.x];
         const int lm8 = A.lam_min & ~7;
         const int nks = (P.n1 - lm8 + 15) >> 4;           // K = 16 steps of the item
@@ -341,8 +358,9 @@ k_joint_fwd_tc(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
     const int sw = row & 7;
     uint32_t tph = 0, zph = 0, d3ph = 0;
     for (int it = blockIdx.x; it < args.n_items; it += gridDim.x) {
-      const int4 item = args.items[it % args.n_base];
-      const int a = item.x, b = it / args.n_base, m0 = item.y;
+      int b;
+      const int4 item = tc_item(args, it, b);
+      const int a = item.x, m0 = item.y;
       bool ok = !abort_flag;
       for (int j = 0; j < item.z && ok; ++j) {
         if (!mbar_wait(&tfull, tph, wait_budget)) { fail(14); ok = false; break; }
@@ -390,7 +408,7 @@ k_joint_fwd_tc(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
       d3ph ^= 1;
       tc_fence_after();
       const int r = m0 + row;
-      float* out = args.P + (((size_t)b * args.n2 + a) * args.n_rows + r) * args.nt;
+      float* out = tc_partial(args, item.w) + (((size_t)b * args.n2 + a) * args.n_rows + r) * args.nt;
 #pragma unroll
       for (int c = 0; c < NT; c += 16) {
         float v[16];
@@ -943,8 +961,9 @@ k_joint_fwd_tp(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
       int armed_a = -1;
       bool ok = true;
       for (int it = blockIdx.x; it < args.n_items && ok && !abort_flag; it += gridDim.x) {
-        const int4 item = args.items[it % args.n_base];
-        const int a = item.x, b = it / args.n_base, m0 = item.y, ntiles = item.z;
+        int b;
+        const int4 item = tc_item(args, it, b);
+        const int a = item.x, m0 = item.y, ntiles = item.z;
         const Rate2 A = P.rates2[a];
         const int lm8 = A.lam_min & ~7;
         const int nkb = (((P.n1 - lm8 + 15) >> 4) + 1) >> 1;
@@ -972,7 +991,7 @@ k_joint_fwd_tp(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
                 if (!RES)
                   tma_load_2d(st + (pl * 2 + part) * kAPlane, &maps.w[pl * 2 + part],
                               lm8 + kb * kBK, m0, &full_bar[stage]);
-                tma_load_3d(sb + (pl * 2 + part) * kYAtom, &maps.y[pl][a], j * BN,
+                tma_load_3d(sb + (pl * 2 + part) * kYAtom, &maps.y[pl][a], (item.w + j) * BN,
                             lm8 + kb * kBK - A.lam_min, 2 * b + part, &full_bar[stage]);
               }
             }
@@ -984,7 +1003,7 @@ k_joint_fwd_tp(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
           armed_w |= 1u << ws;
           armed_w_par = (armed_w_par & ~(1u << ws)) | (wph << ws);
           for (int pl = 0; pl < PS; ++pl)
-            tma_load_2d(sWt + (ws * PS + pl) * kWHalf, &maps.wt[pl], j * BN, a * NT, &wfull[ws]);
+            tma_load_2d(sWt + (ws * PS + pl) * kWHalf, &maps.wt[pl], (item.w + j) * BN, a * NT, &wfull[ws]);
           if (++ws == WS) { ws = 0; wph ^= 1; }
         }
       }
@@ -1003,7 +1022,8 @@ k_joint_fwd_tp(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
       uint32_t phase = 0, tph = 0, aph = 0, par = 0;
       bool ok = true;
       for (int it = blockIdx.x; it < args.n_items && ok && !abort_flag; it += gridDim.x) {
-        const int4 item = args.items[it % args.n_base];
+        int b;
+        const int4 item = tc_item(args, it, b);
         const Rate2 A = P.rates2[item.x];
         const int lm8 = A.lam_min & ~7;
         const int nks = (P.n1 - lm8 + 15) / 16;
@@ -1068,7 +1088,8 @@ k_joint_fwd_tp(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
       uint32_t sph = 0, wph = 0, dph = 0, tiles = 0;
       bool ok = true;
       for (int it = blockIdx.x; it < args.n_items && ok && !abort_flag; it += gridDim.x) {
-        const int4 item = args.items[it % args.n_base];
+        int b;
+        const int4 item = tc_item(args, it, b);
         // the epilogue has read the previous item's accumulators
         if (!mbar_wait(&dfree, dph ^ 1, wait_budget)) { fail(36); ok = false; break; }
         dph ^= 1;
@@ -1117,8 +1138,9 @@ k_joint_fwd_tp(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
     const uint32_t t_zw = t_z + lane_off + cg * 8;
     uint32_t tph = 0, sph = 0, dph = 0;
     for (int it = blockIdx.x; it < args.n_items; it += gridDim.x) {
-      const int4 item = args.items[it % args.n_base];
-      const int a = item.x, b = it / args.n_base, m0 = item.y;
+      int b;
+      const int4 item = tc_item(args, it, b);
+      const int a = item.x, m0 = item.y;
       bool ok = !abort_flag;
       for (int j = 0; j < item.z && ok; ++j) {
         if (!mbar_wait(&tfull, tph, wait_budget)) { fail(39); ok = false; break; }
@@ -1247,7 +1269,7 @@ k_joint_fwd_tp(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
       const int lam = spin ? r - p * P.n1 : r - args.pr_phi0;
       if (r < args.n_rows && (spin || r >= args.pr_phi0) && (d == 0 || spin)) {
         const int crow = (d == 0 ? (p < P.n_fr ? p : 2 * P.n_fr) : p + P.n_fr) * P.n1 + lam;
-        float* out = args.P + ((size_t)b * args.n2 + a) * (size_t)P.C * P.n1 * args.nt +
+        float* out = tc_partial(args, item.w) + ((size_t)b * args.n2 + a) * (size_t)P.C * P.n1 * args.nt +
                      (size_t)crow * args.nt;
         if (args.nt == NT) {
 #pragma unroll
@@ -1278,54 +1300,69 @@ constexpr int kPoolThreads = 256;
 constexpr int kPoolRowsMax = 8192;   // n1 * n_t floats staged per channel
 
 __global__ void __launch_bounds__(kPoolThreads)
-k_pool_lambda(DevPlan Pd, const float* __restrict__ P, float* __restrict__ s2) {
+k_pool_lambda(DevPlan Pd, const float* __restrict__ P, const float* __restrict__ P2,
+              long long part_stride, int part_samples, float* __restrict__ s2) {
   pdl_enter();
   __shared__ float rows[kPoolRowsMax];
   __shared__ float phi[1024];
   const int a = blockIdx.x, b = blockIdx.y;
+  const int c0 = Pd.C * blockIdx.z / gridDim.z, c1 = Pd.C * (blockIdx.z + 1) / gridDim.z;
   const int n1 = Pd.n1, nt = Pd.n_t, nfm = Pd.N_fr - 1, C = Pd.C;
   const Rate2 A = Pd.rates2[a];
   const int nout = Pd.n_lo * nt, nrow = n1 * nt;
   float* out0 = s2 + (size_t)b * Pd.s2_stride + (size_t)a * C * Pd.n_lo * nt;
-  const float* in0 = P + ((size_t)b * Pd.n2 + a) * (size_t)(C * n1) * nt;
+  const size_t base0 = ((size_t)b * Pd.n2 + a) * (size_t)(C * n1) * nt;
+  // the rows of the rate's parts, summed in their order
+  const int parts = (A.L + part_samples - 1) / part_samples;
+  auto in = [&](size_t i) {
+    float v = P[base0 + i];
+    for (int q = 1; q < parts; ++q) v += P2[(q - 1) * (size_t)part_stride + base0 + i];
+    return v;
+  };
+  // a channel's rows into registers, every load of a part in flight at once
+  constexpr int kPer = kPoolRowsMax / kPoolThreads;   // staged floats per thread
+  float nxt[kPer];
+  auto load = [&](int c) {
+    const size_t r0 = base0 + (size_t)c * nrow;
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) {
+      const int i = threadIdx.x + q * kPoolThreads;
+      nxt[q] = i < nrow ? P[r0 + i] : 0.f;
+    }
+    for (int u = 1; u < parts; ++u) {
+      const float* pu = P2 + (u - 1) * (size_t)part_stride + r0;
+#pragma unroll
+      for (int q = 0; q < kPer; ++q) {
+        const int i = threadIdx.x + q * kPoolThreads;
+        if (i < nrow) nxt[q] += pu[i];
+      }
+    }
+  };
   if (A.s == 0 || !Pd.average_fr || nrow > kPoolRowsMax || Pd.N_fr > 1024) {
-    for (int c = 0; c < C; ++c) {
+    for (int c = c0; c < c1; ++c) {
       float* out = out0 + (size_t)c * nout;
-      const float* in = in0 + (size_t)c * nrow;
+      const size_t r0 = (size_t)c * nrow;
       for (int i = threadIdx.x; i < nout; i += blockDim.x) {
         if (A.s == 0) { out[i] = 0.f; continue; }
-        if (!Pd.average_fr) { out[i] = in[i]; continue; }
+        if (!Pd.average_fr) { out[i] = in(r0 + i); continue; }
         const int lo = i / nt, t = i % nt;
         float v = 0.f;
-        for (int r = 0; r < n1; ++r) v += __ldg(&Pd.phiF[(lo * Pd.s_F - r) & nfm]) * in[r * nt + t];
+        for (int r = 0; r < n1; ++r) v += __ldg(&Pd.phiF[(lo * Pd.s_F - r) & nfm]) * in(r0 + r * nt + t);
         out[i] = v;
       }
     }
     return;
   }
   for (int i = threadIdx.x; i < Pd.N_fr; i += blockDim.x) phi[i] = __ldg(&Pd.phiF[i]);
-  constexpr int kPer = kPoolRowsMax / kPoolThreads;   // staged floats per thread
-  float nxt[kPer];
-#pragma unroll
-  for (int q = 0; q < kPer; ++q) {
-    const int i = threadIdx.x + q * kPoolThreads;
-    nxt[q] = i < nrow ? in0[i] : 0.f;
-  }
-  for (int c = 0; c < C; ++c) {
+  load(c0);
+  for (int c = c0; c < c1; ++c) {
 #pragma unroll
     for (int q = 0; q < kPer; ++q) {
       const int i = threadIdx.x + q * kPoolThreads;
       if (i < nrow) rows[i] = nxt[q];
     }
     __syncthreads();
-    if (c + 1 < C) {
-      const float* in = in0 + (size_t)(c + 1) * nrow;
-#pragma unroll
-      for (int q = 0; q < kPer; ++q) {
-        const int i = threadIdx.x + q * kPoolThreads;
-        if (i < nrow) nxt[q] = in[i];
-      }
-    }
+    if (c + 1 < c1) load(c + 1);
     float* out = out0 + (size_t)c * nout;
     for (int i = threadIdx.x; i < nout; i += blockDim.x) {
       const int lo = i / nt, t = i - (i / nt) * nt;
@@ -1592,29 +1629,51 @@ jtfs_status build_tc_tables(jtfs_plan* p) {
   p->pr_phi0 = (p->n_fr * p->n1 + 31) / 32 * 32;
   p->n_pr = p->pr_phi0 + p->n1;
   const int tile_n = p->tc_pair ? 64 : BN;
-  struct It { int a, m0, nt; long long cost; };
-  std::vector<It> its;
+  struct It { int a, m0, nt, t0; long long cost; };
   const int rows = p->tc_pair ? p->n_pr : p->C * p->n1;
-  for (int a = 0; a < p->n2; ++a) {
-    const Rate2& A = p->rates2[a];
-    if (A.s == 0) continue;
-    const int ntiles = (A.L + tile_n - 1) / tile_n;
-    const int kblocks = tc_item_kb(p->n1, A.lam_min);
-    for (int m0 = 0; m0 < rows; m0 += kBM) its.push_back({a, m0, ntiles, (long long)ntiles * (kblocks + 2)});
-  }
-  // items whose W tile fits the resident form first, longest first
   const int res_kb = tc_res_kb(p);
-  auto nkb = [&](const It& x) { return tc_item_kb(p->n1, p->rates2[x.a].lam_min); };
-  std::stable_sort(its.begin(), its.end(), [&](const It& x, const It& y) {
-    const bool rx = nkb(x) <= res_kb, ry = nkb(y) <= res_kb;
-    if (rx != ry) return rx;
-    return x.cost > y.cost;
-  });
+  auto nkb = [&](int a) { return tc_item_kb(p->n1, p->rates2[a].lam_min); };
+  int max_tiles = 1;
+  for (const Rate2& A : p->rates2)
+    if (A.s) max_tiles = std::max(max_tiles, (A.L + tile_n - 1) / tile_n);
+  // The longest rates walked whole (level 0), or in 2, 4 or 8 parts of equal numbers of tiles,
+  // whose pooled rows k_pool_lambda adds: a batch too small to fill the SMs with whole rates takes
+  // the first level whose longest item is at most 0.3 of an SM's share of the work (with no more
+  // than 0.3 the last items end close together; more parts cost a W load and a row write each).
+  // N = 2^16, whole rates -> parts: one signal, FP32-grade, contraction forward 272 -> 127 us (8
+  // parts); five, BF16, 732 -> 324 us (4); one signal of 2^12 in the 64-frame form 59 -> 36 us (2).
   p->tc_items.clear();
-  p->tc_n_res = 0;
-  for (auto& it : its) {
-    p->tc_items.push_back(it.a); p->tc_items.push_back(it.m0); p->tc_items.push_back(it.nt); p->tc_items.push_back(0);
-    if (nkb(it) <= res_kb) ++p->tc_n_res;
+  p->tc_levels.clear();
+  for (int parts = 1; parts <= 8 && (parts == 1 || max_tiles >= parts); parts *= 2) {
+    jtfs_plan::TcLevel lv = {};
+    lv.first = (int)(p->tc_items.size() / 4);
+    lv.cap = (max_tiles + parts - 1) / parts;
+    lv.parts = (max_tiles + lv.cap - 1) / lv.cap;
+    std::vector<It> its;
+    for (int a = 0; a < p->n2; ++a) {
+      const Rate2& A = p->rates2[a];
+      if (A.s == 0) continue;
+      const int ntiles = (A.L + tile_n - 1) / tile_n;
+      for (int t0 = 0; t0 < ntiles; t0 += lv.cap)
+        for (int m0 = 0; m0 < rows; m0 += kBM) {
+          const int nt = std::min(lv.cap, ntiles - t0);
+          its.push_back({a, m0, nt, t0, (long long)nt * (nkb(a) + 2)});
+        }
+    }
+    // items whose W tile fits the resident form first, longest first
+    std::stable_sort(its.begin(), its.end(), [&](const It& x, const It& y) {
+      const bool rx = nkb(x.a) <= res_kb, ry = nkb(y.a) <= res_kb;
+      if (rx != ry) return rx;
+      return x.cost > y.cost;
+    });
+    for (auto& it : its) {
+      for (int v : {it.a, it.m0, it.nt, it.t0}) p->tc_items.push_back(v);
+      if (nkb(it.a) <= res_kb) ++lv.n_res;
+      lv.max_cost = std::max(lv.max_cost, it.cost);
+      lv.cost += it.cost;
+    }
+    lv.n = (int)its.size();
+    p->tc_levels.push_back(lv);
   }
   size_t off = 0;
   auto place = [&](size_t bytes) { size_t at = off; off += (bytes + 1023) & ~(size_t)1023; return at; };
@@ -1660,7 +1719,7 @@ jtfs_status build_tc_tables(jtfs_plan* p) {
 }
 
 jtfs_status launch_joint_fwd_tc(const jtfs_plan* p, int B, const void* yhi_v, const void* ylo_v,
-                                float* Pbuf, float* s2, cudaStream_t st) {
+                                float* Pbuf, float* part_buf, float* s2, cudaStream_t st) {
   const DevPlan& d = p->dp;
   TcMaps maps;
   std::string err;
@@ -1722,13 +1781,23 @@ jtfs_status launch_joint_fwd_tc(const jtfs_plan* p, int B, const void* yhi_v, co
       return JTFS_ERR_CUDA;
     }
   }
-  const int n_all = (int)(p->tc_items.size() / 4);
   const bool tp = p->tc_pair;                // the spin-pair form pools on the tensor cores
   const bool f16 = NT == 16 && !tp;          // the 16-frame TF32 form
   auto stages_for = [&](bool res) {
     return tp ? tp_stages_for(p, res) : (f16 ? tc16_stages_for(p, res) : tc_stages_for(p, res));
   };
-  const int n_res = stages_for(true) >= 2 ? p->tc_n_res : 0;
+  int n_sm = 148;
+  cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, p->device);
+  // parts past the first go to part_buf, which holds 2 y_len floats per signal
+  const long long p_unit = (long long)p->n2 * p->C * p->n1 * p->n_t;
+  size_t level = 0;
+  while (part_buf && level + 1 < p->tc_levels.size() &&
+         10 * p->tc_levels[level].max_cost * n_sm > 3 * B * p->tc_levels[level].cost &&
+         (p->tc_levels[level + 1].parts - 1) * p_unit <= 2 * p->y_len)
+    ++level;
+  const jtfs_plan::TcLevel& lv = p->tc_levels[level];
+  const int n_all = lv.n;
+  const int n_res = stages_for(true) >= 2 ? lv.n_res : 0;
   if (n_all > n_res && stages_for(false) < 2) {
     set_error("tensor-core forward: no shared-memory layout for this configuration");
     return JTFS_ERR_UNSUPPORTED;
@@ -1743,12 +1812,14 @@ jtfs_status launch_joint_fwd_tc(const jtfs_plan* p, int B, const void* yhi_v, co
   args.pr_phi0 = p->pr_phi0;
   args.nt = p->n_t;
   args.P = Pbuf;
+  args.P2 = part_buf;
+  args.part_stride = B * p_unit;
+  args.part_tiles = lv.cap;
+  args.split = level > 0;
   args.n2 = p->n2;
   args.err = p->d_err;
   args.wait_ns = p->wait_ns;
   jtfs_status rc;
-  int n_sm = 148;
-  cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, p->device);
 #define JTFS_LAUNCH_TC(NTV, BNV, RESV)                                                          \
   do {                                                                                          \
     if ((rc = cuda_check(cudaFuncSetAttribute(k_joint_fwd_tc<NTV, BNV, RESV>,                 \
@@ -1785,7 +1856,7 @@ jtfs_status launch_joint_fwd_tc(const jtfs_plan* p, int B, const void* yhi_v, co
     const int first = res ? 0 : n_res, count = res ? n_res : n_all - n_res;
     if (count <= 0) continue;
     args.late = pass == 1 && n_res > 0;
-    args.items = reinterpret_cast<const int4*>(p->d_tc_items) + first;
+    args.items = reinterpret_cast<const int4*>(p->d_tc_items) + lv.first + first;
     args.n_base = count;
     args.n_items = count * B;
     args.stages = stages_for(res);
@@ -1811,7 +1882,8 @@ jtfs_status launch_joint_fwd_tc(const jtfs_plan* p, int B, const void* yhi_v, co
 #undef JTFS_LAUNCH_TC16
 #undef JTFS_LAUNCH_PAIR
 #undef JTFS_LAUNCH_TP1
-  launch_pdl(k_pool_lambda, dim3(p->n2, B), kPoolThreads, 0, st, d, Pbuf, s2);
+  launch_pdl(k_pool_lambda, dim3(p->n2, B, channel_split(p, B, n_sm)), kPoolThreads, 0, st, d, Pbuf,
+             part_buf, args.part_stride, args.part_tiles * (p->tc_pair ? 64 : BN), s2);
   ++p->prof.launches;
   return cuda_check(cudaGetLastError(), "k_pool_lambda");
 }

@@ -1573,12 +1573,13 @@ k_g1(DevPlan Pd, const float* __restrict__ gs2, int NT, int g1_rows,
   __shared__ float gin[kG1InMax];
   __shared__ float phi[1024];
   const int a = blockIdx.x, b = blockIdx.y;
+  const int c0 = Pd.C * blockIdx.z / gridDim.z, c1 = Pd.C * (blockIdx.z + 1) / gridDim.z;
   const int n1 = Pd.n1, nt = Pd.n_t, nfm = Pd.N_fr - 1, C = Pd.C;
   const int nin = Pd.average_fr ? Pd.n_lo * nt : n1 * nt;
   const bool staged = nin <= kG1InMax && Pd.N_fr <= 1024;
   if (staged)
     for (int i = threadIdx.x; i < Pd.N_fr; i += blockDim.x) phi[i] = __ldg(&Pd.phiF[i]);
-  for (int c = 0; c < C; ++c) {
+  for (int c = c0; c < c1; ++c) {
     const float* g = gs2 + (size_t)b * Pd.s2_stride + ((size_t)a * C + c) * Pd.n_lo * nt;
     const size_t o0 = ((size_t)(b * Pd.n2 + a) * g1_rows + (size_t)c * n1) * NT;
     if (staged) {
@@ -1621,6 +1622,7 @@ k_g1(DevPlan Pd, const float* __restrict__ gs2, int NT, int g1_rows,
       if (g1lo) *reinterpret_cast<uint4*>(g1lo + o) = make_uint4(lw[0], lw[1], lw[2], lw[3]);
     }
   }
+  if (blockIdx.z) return;
   // the block's padding rows C n1 .. g1_rows - 1 (read by the last chunks' boxes) are zero
   const size_t ob = (size_t)(b * Pd.n2 + a) * g1_rows * NT;
   for (int i = C * n1 * NT + threadIdx.x * 8; i < g1_rows * NT; i += blockDim.x * 8) {
@@ -1865,8 +1867,11 @@ jtfs_status launch_joint_bwd_tc(const jtfs_plan* p, int B, const void* yhi_v, co
   const size_t g1_plane = tcb_g1_bytes(p, B) / 2;
   __nv_bfloat16* g1hi = (__nv_bfloat16*)g1buf;
   __nv_bfloat16* g1lo = (__nv_bfloat16*)((char*)g1buf + g1_plane);
+  int n_sm = 148;
+  cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, p->device);
   // G1 (phi_F adjoint of g_S2), zero padded by the kernel
-  launch_pdl(k_g1, dim3(p->n2, B), kG1Threads, 0, st, d, gs2, NT, g1_rows, g1hi, three ? g1lo : nullptr);
+  launch_pdl(k_g1, dim3(p->n2, B, channel_split(p, B, n_sm)), kG1Threads, 0, st, d, gs2, NT, g1_rows, g1hi,
+             three ? g1lo : nullptr);
   ++p->prof.launches;
   if ((rc = cuda_check(cudaGetLastError(), "k_g1")) != JTFS_OK) return rc;
   std::string err;
@@ -1925,8 +1930,6 @@ jtfs_status launch_joint_bwd_tc(const jtfs_plan* p, int B, const void* yhi_v, co
   args.gy = gy;
   args.err = p->d_err;
   args.wait_ns = p->wait_ns;
-  int n_sm = 148;
-  cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, p->device);
   TbMaps maps;
   for (int i = 0; i < 4; ++i) maps.w[i] = mw[i];
   for (int h = 0; h < 2; ++h) {
