@@ -153,6 +153,10 @@ struct jtfs_plan {
   int tcbf_n1;                 // tcbf_n1 items with K1 <= 64 first
   int tcbf_n2a = 0;            // of the two-atom items, those with K1 <= 96 (first)
   int tcbf_n3 = 0;             // three-atom items (K1 <= 160, spin-pair form), last
+  int tcbf_sub_a0 = 0, tcbf_sub_a1 = 0;   // rates of the three-atom items
+  long long tcbf_sub_off = 0, tcbf_sub_len = 0;   // their range of a signal's packed Y
+  long long tcbf_sub_max = 0;  // room for parts of it at the start of the FP32 Y buffer
+  long long tcbf_cost = 0, tcbf_cost3 = 0;   // of all items of a signal, of a three-atom item
   int* d_tcbf_items;
   std::vector<int> tcb_fb_items;     // (alpha, n0): rates past the tensor-core backward's
   std::vector<int> tcb_fb_rowitems;  // lambda' capacity, on CUDA cores; their Y row items
@@ -259,7 +263,9 @@ bool tcb_supported(const jtfs_plan* p);
 jtfs_status build_tcb_tables(jtfs_plan* p);
 size_t tcb_g1_bytes(const jtfs_plan* p, int64_t B);
 jtfs_status launch_joint_bwd_tc(const jtfs_plan* p, int B, const void* yhi, const void* ylo,
-                                const float* gs2, void* g1buf, float2* gy, cudaStream_t st);
+                                const float* gs2, void* g1buf, float2* gy, float2* part_buf,
+                                cudaStream_t st);
+int tcb_parts(const jtfs_plan* p, int B);
 
 jtfs_status launch_forward(const jtfs_plan* p, const float* x, int B, float* s0, float* s1,
                            float* s2, float* u1, const Workspace& w, cudaStream_t st);

@@ -244,11 +244,18 @@ k_joint_bwd_simt(DevPlan P, const int2* __restrict__ items, const float2* __rest
   }
 }
 
+// Parts 1, 2, ... of the gY rows of the rates [a0, a1) (the tensor-core backward of small batches).
+struct GyParts {
+  const float2* gy2;
+  long long sub_off, sub_len;
+  int a0, a1, parts;
+};
+
 // Spectra of the gY rows, in place: G rows of one rate per CTA (the Y producer's row items),
 // batched forward FFT (padded radix-16 passes, bit-reversed loads), written back in natural
 // order.
 __global__ void __launch_bounds__(kRowBound)
-k_gy_spectra(DevPlan P, const int4* __restrict__ items, float2* __restrict__ gy) {
+k_gy_spectra(DevPlan P, const int4* __restrict__ items, float2* __restrict__ gy, GyParts gp) {
   pdl_enter();
   extern __shared__ float2 sm[];
   const int4 it = items[blockIdx.x];
@@ -260,7 +267,15 @@ k_gy_spectra(DevPlan P, const int4* __restrict__ items, float2* __restrict__ gy)
   // two samples per 16-byte access where the block's rows start 16-byte aligned (rows hold an
   // even number of samples), else one
   const bool pair = L >= 2 && ((uintptr_t)g & 15) == 0;
-  if (pair) {
+  if (gp.parts > 1 && a >= gp.a0 && a < gp.a1) {
+    // rows whose gY was summed in parts
+    const float2* g2 = gp.gy2 + (size_t)b * P.y_len + (A.off_y - gp.sub_off) + (size_t)(lam0 - A.lam_min) * L;
+    for (int idx = threadIdx.x; idx < total; idx += step) {
+      float2 v = g[idx];
+      for (int q = 1; q < gp.parts; ++q) v = cadd(v, g2[(q - 1) * gp.sub_len + idx]);
+      sm[fft_pos(((idx >> logL) << logL) + bitrev(idx & (L - 1), logL), logL)] = v;
+    }
+  } else if (pair) {
     // four 16-byte loads in flight per thread before their shared-memory stores
     const float4* g4 = reinterpret_cast<const float4*>(g);
     const int total2 = total >> 1;
@@ -638,7 +653,7 @@ jtfs_status launch_backward(const jtfs_plan* p, const float* x, const float* u1,
       launch_pdl(k_second_order_rows<1>, dim3((unsigned)(p->rowitems.size() / 4), B), p->row_threads, (size_t)p->rows_cap * 17 / 2, st, d, reinterpret_cast<const int4*>(p->d_rowitems), w.uh, nullptr, (__nv_bfloat16*)w.ybh, (__nv_bfloat16*)w.ybl, B);
     }
     StageScope sc(p, kStJointBwd, st, 0);   // the launcher counts its kernels
-    jtfs_status r2 = launch_joint_bwd_tc(p, B, w.ybh, w.ybl, gs2, w.g1, w.gy, st);
+    jtfs_status r2 = launch_joint_bwd_tc(p, B, w.ybh, w.ybl, gs2, w.g1, w.gy, w.y, st);
     if (r2 != JTFS_OK) return r2;
     if (!p->tcb_fb_items.empty()) {
       // rates beyond the tensor-core backward's lambda' capacity: FP32 Y rows of those rates
@@ -658,10 +673,12 @@ jtfs_status launch_backward(const jtfs_plan* p, const float* x, const float* u1,
   } else if (p->y_len > 0) {
     cudaMemsetAsync(w.gy, 0, (size_t)B * p->y_len * sizeof(float2), st);
   }
+  const GyParts gp = {w.y, p->tcbf_sub_off, p->tcbf_sub_len, p->tcbf_sub_a0, p->tcbf_sub_a1,
+                      gs2 && n_items > 0 && p->use_tcb ? tcb_parts(p, B) : 1};
   {
     StageScope sc(p, kStSecondOrderBwd, st, 2);
     if (!p->rowitems.empty())
-      launch_pdl(k_gy_spectra, dim3((unsigned)(p->rowitems.size() / 4), B), p->row_threads, (size_t)p->rows_cap * 17 / 2, st, d, reinterpret_cast<const int4*>(p->d_rowitems), w.gy);
+      launch_pdl(k_gy_spectra, dim3((unsigned)(p->rowitems.size() / 4), B), p->row_threads, (size_t)p->rows_cap * 17 / 2, st, d, reinterpret_cast<const int4*>(p->d_rowitems), w.gy, gp);
     launch_pdl(k_second_order_bwd, dim3(p->n1, B), 256, (size_t)p->L1max * 17 / 2, st, d, w.gy, gs1, w.gu1);
   }
   {
@@ -705,7 +722,7 @@ jtfs_status launch_scat1d_backward(const jtfs_plan* p, const float* x, const flo
   {
     StageScope sc(p, kStSecondOrderBwd, st, 2);
     if (!p->rowitems.empty())
-      launch_pdl(k_gy_spectra, dim3((unsigned)(p->rowitems.size() / 4), B), p->row_threads, (size_t)p->rows_cap * 17 / 2, st, d, reinterpret_cast<const int4*>(p->d_rowitems), w.gy);
+      launch_pdl(k_gy_spectra, dim3((unsigned)(p->rowitems.size() / 4), B), p->row_threads, (size_t)p->rows_cap * 17 / 2, st, d, reinterpret_cast<const int4*>(p->d_rowitems), w.gy, GyParts{nullptr, 0, 0, 0, 0, 1});
     launch_pdl(k_second_order_bwd, dim3(p->n1, B), 256, (size_t)p->L1max * 17 / 2, st, d, w.gy, gs1, w.gu1);
   }
   {

@@ -1111,8 +1111,9 @@ struct TpMaps {
 struct TpArgs {
   const int4* items;    // (alpha, n0, lambda' start = lam_min & ~7, K1 <= 64) per base
   int n_base;
-  int n_items;
-  int n_chunks;         // ceil(n_pr / 32)
+  int n_items;          // n_base * B * parts
+  int n_chunks;         // ceil(n_pr / RC)
+  int parts;            // an item's chunks split over this many CTAs (small batches)
   int g1_rows;          // rows per (b, alpha) block of G1
   int wbufs;            // W chunk ring depth (2..kPairWBufs)
   int pr_phi0;          // first phi_F pair row (multiple of 32)
@@ -1120,12 +1121,24 @@ struct TpArgs {
   int chan_phi0;        // 2 n_fr n1: channel row of the first phi_F row
   const int* wt_row0;
   float2* gy;
+  float2* gy2;          // parts 1, 2, ...: their gY of rate a, signal b, at b y_len +
+  long long sub_off, sub_len;   // (part - 1) sub_len + off_y - sub_off
   int late;             // 1: independent of the launch before it
   int* err;
   uint64_t wait_ns;     // budget of every barrier wait (the plan's)
 };
 
 constexpr int kPairWBufs = 6;
+
+// item, signal and chunk range [j0, j1) of work item it
+__device__ __forceinline__ int4 pair_item(const TpArgs& args, int it, int& b, int& part, int& j0, int& j1) {
+  const int u = it / args.parts;
+  part = it - u * args.parts;
+  b = u / args.n_base;
+  j0 = args.n_chunks * part / args.parts;
+  j1 = args.n_chunks * (part + 1) / args.parts;
+  return args.items[u - b * args.n_base];
+}
 
 template <int PL, int NAT, int KMV, int RCV, int NT>
 __global__ void __launch_bounds__(kFThreads, 1)
@@ -1214,20 +1227,21 @@ k_joint_bwd_pair(const __grid_constant__ TpMaps maps, TpArgs args, DevPlan P) {
       uint32_t a4_ph = 0;
       bool ok = true;
       for (int it = blockIdx.x; it < args.n_items && ok && !abort_flag; it += gridDim.x) {
-        const int4 item = args.items[it % args.n_base];
-        const int a = item.x, b = it / args.n_base, n0 = item.y, start = item.z, K1 = item.w;
+        int b, part, j0, j1;
+        const int4 item = pair_item(args, it, b, part, j0, j1);
+        const int a = item.x, n0 = item.y, start = item.z, K1 = item.w;
         const Rate2 A = P.rates2[a];
         const int nkb1 = (K1 + 31) / 32;
         if (!mbar_wait(&a1_free, a1_ph ^ 1, wait_budget)) { fail(81); break; }
         mbar_arrive_expect_tx(&a1_full, PL * 2 * 2 * nkb1 * 4096 + (YT ? 0 : PL * kA4Plane));
         armed_a1 = (int)a1_ph;
         for (int pl = 0; pl < PL; ++pl)
-          for (int part = 0; part < 2; ++part)
+          for (int c = 0; c < 2; ++c)   // re, im
             for (int h = 0; h < 2; ++h)
               for (int kb = 0; kb < nkb1; ++kb)
-                tma_load_3d(sA1 + (pl * 2 + part) * kA1Plane + h * KM * 128 + kb * 32 * 128,
+                tma_load_3d(sA1 + (pl * 2 + c) * kA1Plane + h * KM * 128 + kb * 32 * 128,
                             &maps.y[pl][a], n0 + h * 64, start - A.lam_min + kb * 32,
-                            2 * b + part, &a1_full);
+                            2 * b + c, &a1_full);
         a1_ph ^= 1;
         uint64_t* a4_bar = &a1_full;
         if (YT) {
@@ -1243,7 +1257,7 @@ k_joint_bwd_pair(const __grid_constant__ TpMaps maps, TpArgs args, DevPlan P) {
           a4b ^= 1;
         }
         const int g1row = (b * P.n2 + a) * args.g1_rows;
-        for (int j = 0; j < args.n_chunks; ++j) {
+        for (int j = j0; j < j1; ++j) {
           if (!mbar_wait(&w_empty[wst], wph ^ 1, wait_budget)) { fail(82); ok = false; break; }
           mbar_arrive_expect_tx(&w_full[wst], kWBuf);
           armed_w |= 1u << wst;
@@ -1282,13 +1296,13 @@ k_joint_bwd_pair(const __grid_constant__ TpMaps maps, TpArgs args, DevPlan P) {
       int wst = 0, a4b = 0;
       bool ok = true;
       for (int it = blockIdx.x; it < args.n_items && ok && !abort_flag; it += gridDim.x) {
-        const int4 item = args.items[it % args.n_base];
-        const int nks1 = item.w / 16;
+        int b, part, j0, j1;
+        const int nks1 = pair_item(args, it, b, part, j0, j1).w / 16;
         if (!mbar_wait(YT ? &yt_full : &a1_full, a1_ph, wait_budget)) { fail(83); break; }
         a1_ph ^= 1;
         if (YT && !mbar_wait(&a4_full[a4b], a4_ph, wait_budget)) { fail(93); break; }
         const uint32_t a1 = smem_u32(sA1), a4 = smem_u32(sA4 + a4b * PL * kA4Plane);
-        for (int j = 0; j < args.n_chunks && ok; ++j) {
+        for (int j = j0; j < j1 && ok; ++j) {
           if (!mbar_wait(&w_full[wst], wph, wait_budget)) { fail(84); ok = false; break; }
           if (!mbar_wait(&d1_free, d1f_ph ^ 1, wait_budget)) { fail(85); ok = false; break; }
           d1f_ph ^= 1;
@@ -1351,11 +1365,13 @@ k_joint_bwd_pair(const __grid_constant__ TpMaps maps, TpArgs args, DevPlan P) {
       int wst = 0;
       bool ok = true;
       for (int it = blockIdx.x; it < args.n_items && ok && !abort_flag; it += gridDim.x) {
-        for (int j = 0; j < args.n_chunks && ok; ++j) {
+        int b, part, j0, j1;
+        pair_item(args, it, b, part, j0, j1);
+        for (int j = j0; j < j1 && ok; ++j) {
           if (!mbar_wait(&a2_full, a2_ph, wait_budget)) { fail(86); ok = false; break; }
           a2_ph ^= 1;
           if (!mbar_wait(&w_full[wst], wph, wait_budget)) { fail(87); ok = false; break; }
-          if (j == 0) {
+          if (j == j0) {
             if (!mbar_wait(&d2_free, d2f_ph ^ 1, wait_budget)) { fail(88); ok = false; break; }
             d2f_ph ^= 1;
           }
@@ -1371,7 +1387,7 @@ k_joint_bwd_pair(const __grid_constant__ TpMaps maps, TpArgs args, DevPlan P) {
               const uint32_t wo = q * NAT * 2 * kWBlk + ks * 2048;
               const uint64_t wr = dW + (uint64_t)(wo >> 4);
               const uint64_t wi = dW + (uint64_t)((wo + kWBlk) >> 4);
-              const uint32_t f = (j == 0 && ks == 0 && q == 0) ? 0u : 1u;
+              const uint32_t f = (j == j0 && ks == 0 && q == 0) ? 0u : 1u;
               const uint32_t ta = t_a2 + ks * 8;
               mma_f16_ta(t_re, ta, wr, id2, f);
               mma_f16_ta(t_re, ta + RC, wi, id2, 1u);
@@ -1400,7 +1416,9 @@ k_joint_bwd_pair(const __grid_constant__ TpMaps maps, TpArgs args, DevPlan P) {
     // YT: this warp's 32 samples of plane cg of an item's Y^T tile (shared memory, [lambda'][64
     // samples] rows of 128 swizzled bytes) into TMEM, sample n in lane n, two lambda' per column.
     // The caller has seen the last first product of the item before complete.
-    auto stage_y = [&](int nks1) -> bool {
+    auto stage_y = [&](int it) -> bool {
+      int b, part, j0, j1;
+      const int nks1 = pair_item(args, it, b, part, j0, j1).w / 16;
       if (!mbar_wait(&a1_full, y_ph, wait_budget)) { fail(94); return false; }
       y_ph ^= 1;
       tc_fence_after();
@@ -1431,12 +1449,13 @@ k_joint_bwd_pair(const __grid_constant__ TpMaps maps, TpArgs args, DevPlan P) {
       return true;
     };
     bool staged = true;
-    if (YT && (int)blockIdx.x < args.n_items) staged = stage_y(args.items[blockIdx.x % args.n_base].w / 16);
+    if (YT && (int)blockIdx.x < args.n_items) staged = stage_y((int)blockIdx.x);
     for (int it = blockIdx.x; it < args.n_items; it += gridDim.x) {
-      const int4 item = args.items[it % args.n_base];
-      const int a = item.x, b = it / args.n_base, n0 = item.y, start = item.z;
+      int b, part, j0, j1;
+      const int4 item = pair_item(args, it, b, part, j0, j1);
+      const int a = item.x, n0 = item.y, start = item.z;
       bool ok = !abort_flag && staged;
-      for (int j = 0; j < args.n_chunks && ok; ++j) {
+      for (int j = j0; j < j1 && ok; ++j) {
         if (!mbar_wait(&d1_full, d1_ph, wait_budget)) { fail(89); ok = false; break; }
         d1_ph ^= 1;
         tc_fence_after();
@@ -1522,14 +1541,16 @@ k_joint_bwd_pair(const __grid_constant__ TpMaps maps, TpArgs args, DevPlan P) {
       if (!ok) break;
       // the next item's Y^T before this item's results: its first product runs meanwhile
       if (YT && it + (int)gridDim.x < args.n_items)
-        staged = stage_y(args.items[(it + (int)gridDim.x) % args.n_base].w / 16);
+        staged = stage_y(it + (int)gridDim.x);
       // gY of this tile: lambda' = start + c for c in [16 cg, 16 cg + 16)
       if (!mbar_wait(&d2_full, d2_ph, wait_budget)) { fail(91); break; }
       d2_ph ^= 1;
       tc_fence_after();
       const Rate2 A = P.rates2[a];
       const int n = n0 + row;
-      float2* go = args.gy + (size_t)b * P.y_len + A.off_y;
+      float2* go = part == 0 ? args.gy + (size_t)b * P.y_len + A.off_y
+                             : args.gy2 + (size_t)b * P.y_len + (part - 1) * args.sub_len +
+                                   (A.off_y - args.sub_off);
 #pragma unroll
       for (int at = 0; at < NAT; ++at) {      // one atom at a time (registers)
         float vr[16], vi[16];
@@ -1719,6 +1740,19 @@ static bool tcb_rate_fits(const jtfs_plan* p, int a, bool pair_forms) {
 
 bool tcb_supported(const jtfs_plan* p) { return tc_nt(p->n_t) <= 64; }
 
+// CTAs per three-atom item: its chunks are the longest serial chain of the backward (201 us of the
+// 310 us contraction backward of one signal at N = 2^16), so a batch whose share per SM is less
+// than four such items splits them.
+int tcb_parts(const jtfs_plan* p, int B) {
+  int n_sm = 148;
+  cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, p->device);
+  int parts = 1;
+  while (parts < 8 && 4 * p->tcbf_cost3 * n_sm > parts * p->tcbf_cost * B &&
+         (2 * parts - 1) * p->tcbf_sub_len <= p->tcbf_sub_max)
+    parts *= 2;
+  return p->tcbf_n3 > 0 ? parts : 1;
+}
+
 jtfs_status build_tcb_tables(jtfs_plan* p) {
   const int NT = tc_nt(p->n_t);
   std::vector<int> row0(p->n2);
@@ -1785,6 +1819,33 @@ jtfs_status build_tcb_tables(jtfs_plan* p) {
     }
   p->tcbf_n1 = (int)fast1.size();
   p->tcbf_n3 = (int)fast3.size();
+  // The three-atom rates are neighbours (lambda' ranges widen with alpha): parts of their items
+  // past the first keep their gY packed in the FP32 Y buffer, up to the rates that run on CUDA
+  // cores and need their Y rows there.
+  p->tcbf_sub_off = p->tcbf_sub_len = p->tcbf_sub_max = 0;
+  p->tcbf_cost = p->tcbf_cost3 = 0;
+  p->tcbf_sub_a0 = p->tcbf_sub_a1 = 0;
+  if (!fast3.empty()) {
+    int a0 = p->n2, a1 = 0;
+    for (auto& i : fast3) {
+      a0 = std::min(a0, i.a);
+      a1 = std::max(a1, i.a + 1);
+    }
+    long long room = p->y_len, end = 0;
+    for (size_t i = 0; i < p->tcb_fb_items.size(); i += 2)
+      room = std::min(room, p->rates2[p->tcb_fb_items[i]].off_y);
+    for (int a = a0; a < a1; ++a)
+      if (p->rates2[a].s) end = p->rates2[a].off_y + (long long)p->rates2[a].K * p->rates2[a].L;
+    p->tcbf_sub_a0 = a0;
+    p->tcbf_sub_a1 = a1;
+    p->tcbf_sub_off = p->rates2[a0].off_y;
+    p->tcbf_sub_len = end - p->tcbf_sub_off;
+    p->tcbf_sub_max = room;
+  }
+  // costs in K steps: a three-atom item's chunks hold half the rows at about 0.6 of the time each
+  for (auto* v : {&fast1, &fast2, &fast3})
+    for (auto& i : *v) p->tcbf_cost += v == &fast3 ? i.K1 * 5 / 4 : i.K1;
+  for (auto& i : fast3) p->tcbf_cost3 = std::max<long long>(p->tcbf_cost3, i.K1 * 5 / 4);
   // items whose Y^T tile fits the resident three-pass form (K1 <= 96) first, longest first
   std::stable_sort(its.begin(), its.end(), [](const It& x, const It& y) {
     const bool rx = x.K1 <= 96, ry = y.K1 <= 96;
@@ -1856,7 +1917,8 @@ size_t tcb3_smem_bytes(int NT) {
 }
 
 jtfs_status launch_joint_bwd_tc(const jtfs_plan* p, int B, const void* yhi_v, const void* ylo_v,
-                                const float* gs2, void* g1buf, float2* gy, cudaStream_t st) {
+                                const float* gs2, void* g1buf, float2* gy, float2* part_buf,
+                                cudaStream_t st) {
   const DevPlan& d = p->dp;
   const int NT = tc_nt(p->n_t);
   const int rows = p->C * p->n1;
@@ -1984,6 +2046,9 @@ jtfs_status launch_joint_bwd_tc(const jtfs_plan* p, int B, const void* yhi_v, co
       pa.chan_phi0 = 2 * p->n_fr * p->n1;
       pa.wt_row0 = p->d_wtb_row0;
       pa.gy = gy;
+      pa.gy2 = part_buf;
+      pa.sub_off = p->tcbf_sub_off;
+      pa.sub_len = p->tcbf_sub_len;
       pa.err = p->d_err;
       pa.wait_ns = p->wait_ns;
 #define JTFS_LAUNCH_TCBP1(PLV, NATV, KMV, RCV, NTV)                                             \
@@ -2013,7 +2078,8 @@ jtfs_status launch_joint_bwd_tc(const jtfs_plan* p, int B, const void* yhi_v, co
         }
         pa.items = reinterpret_cast<const int4*>(p->d_tcbf_items) + f0;
         pa.n_base = cnt;
-        pa.n_items = cnt * B;
+        pa.parts = nat == 3 ? tcb_parts(p, B) : 1;
+        pa.n_items = cnt * B * pa.parts;
         pa.wbufs = wbp;
         pa.late = launched++ > 0;
         const int grid = std::min(pa.n_items, n_sm);
