@@ -334,7 +334,8 @@ static size_t sob_smem(const jtfs_plan* p) {
 // g_U1 row lambda': sum over rates alpha of the adjoint of psi2 (the gY row's spectrum / Lr
 // times psi-hat_alpha on the row's positive bins), then Re of the inverse row DFT, plus S1's
 // adjoint.
-__global__ void __launch_bounds__(256, 3)   // launched with 256 threads; three blocks per SM
+template <int TH>   // threads: three 256-thread blocks per SM, or one of 512
+__global__ void __launch_bounds__(TH, TH == kRowLaunch ? 3 : 1)
 k_second_order_bwd(DevPlan P, int table, const float2* __restrict__ gys,
                    const float* __restrict__ gs1, float* __restrict__ gu1) {
   pdl_enter();
@@ -430,7 +431,8 @@ k_second_order_bwd(DevPlan P, int table, const float2* __restrict__ gys,
   for (int m = threadIdx.x; m < R.L; m += blockDim.x) out[m] = tmp[fft_pos(m, R.logL)].x;
 }
 
-__global__ void __launch_bounds__(kRowLaunch, 3)   // three 256-thread blocks per SM
+template <int TH>   // threads: three 256-thread blocks per SM, or one of 512
+__global__ void __launch_bounds__(TH, TH == kRowLaunch ? 3 : 1)
 k_stage1_bwd(DevPlan P, const float2* __restrict__ xh, const float* __restrict__ gu1,
              float2* __restrict__ gf) {
   pdl_enter();
@@ -506,7 +508,8 @@ __global__ void k_gxh(DevPlan P, const float2* __restrict__ gf, const float* __r
 
 // g_x[r + D m] = Re(sum_k' e^{2 pi i k' m / M} sum_q H[k' + q M] e^{2 pi i (k' + q M) r / N})
 // (S0's adjoint is already in H unless phi-hat reaches the Nyquist bin)
-__global__ void __launch_bounds__(kFftThreads, 2)   // two 512-thread blocks per SM
+template <int TH>   // threads: two 512-thread blocks per SM, or one of 1024
+__global__ void __launch_bounds__(TH, TH == kFftThreads ? 2 : 1)
 k_gx(DevPlan P, const float2* __restrict__ gxh, const float* __restrict__ gs0, float* __restrict__ gx) {
   pdl_enter();
   extern __shared__ float2 sm[];
@@ -612,8 +615,11 @@ jtfs_status set_attrs(const jtfs_plan* p) {
   const int big = 227 * 1024;
   const void* fns[] = {(const void*)k_uh_from_u1, (const void*)k_joint_bwd_simt<32>,
                        (const void*)k_joint_bwd_simt<16>,
-                       (const void*)k_second_order_bwd, (const void*)k_stage1_bwd,
-                       (const void*)k_gx, (const void*)k_xfft_sub};
+                       (const void*)k_second_order_bwd<kRowLaunch>,
+                       (const void*)k_second_order_bwd<2 * kRowLaunch>,
+                       (const void*)k_stage1_bwd<kRowLaunch>, (const void*)k_stage1_bwd<2 * kRowLaunch>,
+                       (const void*)k_gx<kFftThreads>, (const void*)k_gx<2 * kFftThreads>,
+                       (const void*)k_xfft_sub<kFftThreads>, (const void*)k_xfft_sub<2 * kFftThreads>};
   for (const void* f : fns) {
     jtfs_status st = cuda_check(
         cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, big), "attr");
@@ -646,6 +652,27 @@ static void launch_joint_bwd_simt(const jtfs_plan* p, int n_items, const int* it
   launch_pdl(kernel, dim3((unsigned)n_items, B, wide ? 1 : 2), l.threads, (size_t)l.total * 4, st, p->dp, reinterpret_cast<const int2*>(items), y, gs2, gy);
 }
 
+static void launch_second_order_bwd(const jtfs_plan* p, int B, const float2* gys, const float* gs1,
+                                    float* gu1, cudaStream_t st) {
+  const bool few = few_blocks(p, (long long)p->n1 * B);
+  launch_pdl(few ? k_second_order_bwd<2 * kRowLaunch> : k_second_order_bwd<kRowLaunch>, dim3(p->n1, B),
+             few ? 2 * kRowLaunch : kRowLaunch, sob_smem(p), st, p->dp, (int)sob_table(p), gys, gs1, gu1);
+}
+
+static void launch_stage1_bwd(const jtfs_plan* p, int B, const float2* xh, const float* gu1, float2* gf,
+                              cudaStream_t st) {
+  const bool few = few_blocks(p, (long long)p->n1 * B);
+  launch_pdl(few ? k_stage1_bwd<2 * kRowLaunch> : k_stage1_bwd<kRowLaunch>, dim3(p->n1, B),
+             few ? 2 * kRowLaunch : kRowLaunch, (size_t)p->L1max * 17 / 2, st, p->dp, xh, gu1, gf);
+}
+
+static void launch_gx(const jtfs_plan* p, int B, const float2* gxh, const float* gs0, float* gx,
+                      cudaStream_t st) {
+  const bool few = few_blocks(p, (long long)p->dp.D * B);
+  launch_pdl(few ? k_gx<2 * kFftThreads> : k_gx<kFftThreads>, dim3(p->dp.D, B),
+             few ? 2 * kFftThreads : kFftThreads, (size_t)p->dp.M * 17 / 2, st, p->dp, gxh, gs0, gx);
+}
+
 bool backward_reuses_forward(const jtfs_plan* p) {
   // the forward's BF16 Y planes are the backward's operands (not for TF32, whose forward
   // writes FP32 planes)
@@ -664,7 +691,7 @@ jtfs_status launch_backward(const jtfs_plan* p, const float* x, const float* u1,
   if (!fused) {
     {
       StageScope sc(p, kStXfft, st, 2);
-      launch_pdl(k_xfft_sub, dim3(d.D, B), kFftThreads, (size_t)d.M * 17 / 2, st, d, x, w.xsub);
+      launch_xfft_sub(p, B, x, w.xsub, st);
       launch_pdl(k_xfft_combine, dim3((p->N / 2 + 255) / 256, B), 256, 0, st, d, w.xsub, w.xh);
     }
     {
@@ -705,16 +732,16 @@ jtfs_status launch_backward(const jtfs_plan* p, const float* x, const float* u1,
     StageScope sc(p, kStSecondOrderBwd, st, 2);
     if (!p->rowitems.empty())
       launch_pdl(k_gy_spectra, dim3((unsigned)(p->rowitems.size() / 4), B), p->row_threads, (size_t)p->rows_cap * 17 / 2, st, d, reinterpret_cast<const int4*>(p->d_rowitems), w.gy, gp);
-    launch_pdl(k_second_order_bwd, dim3(p->n1, B), 256, sob_smem(p), st, d, (int)sob_table(p), w.gy, gs1, w.gu1);
+    launch_second_order_bwd(p, B, w.gy, gs1, w.gu1, st);
   }
   {
     StageScope sc(p, kStStage1Bwd, st, 1);
-    launch_pdl(k_stage1_bwd, dim3(p->n1, B), kRowLaunch, (size_t)p->L1max * 17 / 2, st, d, w.xh, w.gu1, w.gf);
+    launch_stage1_bwd(p, B, w.xh, w.gu1, w.gf, st);
   }
   {
     StageScope sc(p, kStGx, st, 2);
     launch_pdl(k_gxh, dim3((p->N / 2 + 255) / 256, B), 256, 0, st, d, w.gf, gs0, w.gxh);
-    launch_pdl(k_gx, dim3(d.D, B), kFftThreads, (size_t)d.M * 17 / 2, st, d, w.gxh, gs0, gx);
+    launch_gx(p, B, w.gxh, gs0, gx, st);
   }
   return cuda_check(cudaGetLastError(), "backward launch");
 }
@@ -729,7 +756,7 @@ jtfs_status launch_scat1d_backward(const jtfs_plan* p, const float* x, const flo
   const DevPlan& d = p->dp;
   {
     StageScope sc(p, kStXfft, st, 2);
-    launch_pdl(k_xfft_sub, dim3(d.D, B), kFftThreads, (size_t)d.M * 17 / 2, st, d, x, w.xsub);
+    launch_xfft_sub(p, B, x, w.xsub, st);
     launch_pdl(k_xfft_combine, dim3((p->N / 2 + 255) / 256, B), 256, 0, st, d, w.xsub, w.xh);
   }
   {
@@ -749,16 +776,16 @@ jtfs_status launch_scat1d_backward(const jtfs_plan* p, const float* x, const flo
     StageScope sc(p, kStSecondOrderBwd, st, 2);
     if (!p->rowitems.empty())
       launch_pdl(k_gy_spectra, dim3((unsigned)(p->rowitems.size() / 4), B), p->row_threads, (size_t)p->rows_cap * 17 / 2, st, d, reinterpret_cast<const int4*>(p->d_rowitems), w.gy, GyParts{nullptr, 0, 0, 0, 0, 1});
-    launch_pdl(k_second_order_bwd, dim3(p->n1, B), 256, sob_smem(p), st, d, (int)sob_table(p), w.gy, gs1, w.gu1);
+    launch_second_order_bwd(p, B, w.gy, gs1, w.gu1, st);
   }
   {
     StageScope sc(p, kStStage1Bwd, st, 1);
-    launch_pdl(k_stage1_bwd, dim3(p->n1, B), kRowLaunch, (size_t)p->L1max * 17 / 2, st, d, w.xh, w.gu1, w.gf);
+    launch_stage1_bwd(p, B, w.xh, w.gu1, w.gf, st);
   }
   {
     StageScope sc(p, kStGx, st, 2);
     launch_pdl(k_gxh, dim3((p->N / 2 + 255) / 256, B), 256, 0, st, d, w.gf, gs0, w.gxh);
-    launch_pdl(k_gx, dim3(d.D, B), kFftThreads, (size_t)d.M * 17 / 2, st, d, w.gxh, gs0, gx);
+    launch_gx(p, B, w.gxh, gs0, gx, st);
   }
   return cuda_check(cudaGetLastError(), "time scattering backward");
 }

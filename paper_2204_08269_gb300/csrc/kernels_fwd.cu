@@ -77,7 +77,8 @@ k_s0(DevPlan P, const float* __restrict__ x, float* __restrict__ s0) {
   }
 }
 
-__global__ void __launch_bounds__(kRowLaunch, 3)   // three 256-thread blocks per SM
+template <int TH>   // threads: three 256-thread blocks per SM, or one of 512
+__global__ void __launch_bounds__(TH, TH == kRowLaunch ? 3 : 1)
 k_scalogram(DevPlan P, const float2* __restrict__ xh, float* __restrict__ u1,
             float2* __restrict__ uh, float* __restrict__ s1) {
   pdl_enter();
@@ -134,6 +135,14 @@ k_scalogram(DevPlan P, const float2* __restrict__ xh, float* __restrict__ u1,
       if (l == 0) s1[((size_t)b * P.n1 + lam) * P.n_t + t] = acc / (float)R.L;
     }
   }
+}
+
+static void launch_scalogram(const jtfs_plan* p, int B, const float2* xh, float* u1, float2* uh,
+                             float* s1, cudaStream_t st) {
+  const bool few = few_blocks(p, (long long)p->n1 * B);
+  launch_pdl(few ? k_scalogram<2 * kRowLaunch> : k_scalogram<kRowLaunch>, dim3(p->n1, B),
+             few ? 2 * kRowLaunch : kRowLaunch, (size_t)p->L1max * 17 / 2 + (size_t)p->L1max * 4, st,
+             p->dp, xh, u1, uh, s1);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -413,8 +422,9 @@ jtfs_status set_attrs(const jtfs_plan* p) {
   if (g_attrs_set[p->device]) return JTFS_OK;
   const int big = 227 * 1024;
   jtfs_status st;
-  if ((st = cuda_check(cudaFuncSetAttribute(k_xfft_sub, cudaFuncAttributeMaxDynamicSharedMemorySize, big), "attr")) != JTFS_OK) return st;
-  if ((st = cuda_check(cudaFuncSetAttribute(k_scalogram, cudaFuncAttributeMaxDynamicSharedMemorySize, big), "attr")) != JTFS_OK) return st;
+  for (const void* f : {(const void*)k_xfft_sub<kFftThreads>, (const void*)k_xfft_sub<2 * kFftThreads>,
+                        (const void*)k_scalogram<kRowLaunch>, (const void*)k_scalogram<2 * kRowLaunch>})
+    if ((st = cuda_check(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, big), "attr")) != JTFS_OK) return st;
   // the row producer holds at most 2^14 complex samples (padded one per 16) next to its
   // static row tables
   const int rows_smem = 140 * 1024;
@@ -526,7 +536,7 @@ jtfs_status launch_scat1d_forward(const jtfs_plan* p, const float* x, int B, flo
   const DevPlan& d = p->dp;
   {
     StageScope sc(p, kStXfft, st, 2);
-    launch_pdl(k_xfft_sub, dim3(d.D, B), kFftThreads, (size_t)d.M * 17 / 2, st, d, x, w.xsub);
+    launch_xfft_sub(p, B, x, w.xsub, st);
     launch_pdl(k_xfft_combine, dim3((p->N / 2 + 255) / 256, B), 256, 0, st, d, w.xsub, w.xh);
   }
   {
@@ -535,7 +545,7 @@ jtfs_status launch_scat1d_forward(const jtfs_plan* p, const float* x, int B, flo
   }
   {
     StageScope sc(p, kStScalogram, st, 1);
-    launch_pdl(k_scalogram, dim3(p->n1, B), kRowLaunch, (size_t)p->L1max * 17 / 2 + (size_t)p->L1max * 4, st, d, w.xh, u1, w.uh, s1);
+    launch_scalogram(p, B, w.xh, u1, w.uh, s1, st);
   }
   if ((rc = cuda_check(cudaMemsetAsync(s2t, 0, (size_t)B * p->n2 * p->n1 * p->n_t * sizeof(float), st), "memset")) != JTFS_OK)
     return rc;
@@ -557,7 +567,7 @@ jtfs_status launch_forward(const jtfs_plan* p, const float* x, int B, float* s0,
   const DevPlan& d = p->dp;
   {
     StageScope sc(p, kStXfft, st, 2);
-    launch_pdl(k_xfft_sub, dim3(d.D, B), kFftThreads, (size_t)d.M * 17 / 2, st, d, x, w.xsub);
+    launch_xfft_sub(p, B, x, w.xsub, st);
     launch_pdl(k_xfft_combine, dim3((p->N / 2 + 255) / 256, B), 256, 0, st, d, w.xsub, w.xh);
   }
   {
@@ -566,7 +576,7 @@ jtfs_status launch_forward(const jtfs_plan* p, const float* x, int B, float* s0,
   }
   {
     StageScope sc(p, kStScalogram, st, 1);
-    launch_pdl(k_scalogram, dim3(p->n1, B), kRowLaunch, (size_t)p->L1max * 17 / 2 + (size_t)p->L1max * 4, st, d, w.xh, u1, w.uh, s1);
+    launch_scalogram(p, B, w.xh, u1, w.uh, s1, st);
   }
   if (p->use_tc && p->cfg.precision == JTFS_PREC_TF32) {
     // TF32 operands: Y as FP32 planes (in the complex FP32 buffer, same size)
@@ -679,10 +689,10 @@ jtfs_status launch_first_order_static(const jtfs_plan* p, const float* x, int B,
   c += a(Bz * p->u1_len * 4);
   float2* uh = (float2*)c;
   const DevPlan& d = p->dp;
-  launch_pdl(k_xfft_sub, dim3(d.D, B), kFftThreads, (size_t)d.M * 17 / 2, st, d, x, xsub);
+  launch_xfft_sub(p, B, x, xsub, st);
   launch_pdl(k_xfft_combine, dim3((p->N / 2 + 255) / 256, B), 256, 0, st, d, xsub, xh);
   launch_pdl(k_s0, dim3(kS0Split * p->n_t, B), kS0Threads, 0, st, d, x, s0);
-  launch_pdl(k_scalogram, dim3(p->n1, B), kRowLaunch, (size_t)p->L1max * 17 / 2 + (size_t)p->L1max * 4, st, d, xh, u1, uh, s1);
+  launch_scalogram(p, B, xh, u1, uh, s1, st);
   return cuda_check(cudaGetLastError(), "first-order static launch");
 }
 

@@ -15,10 +15,20 @@ constexpr int kFftThreads = 512;
 // per-row first-order kernels are launched with 256 threads: with their registers, 512-thread
 // blocks leave one block per SM
 constexpr int kRowLaunch = 256;
+// A batch whose blocks do not even fill the SMs once leaves the time to the longest row: those
+// launches take twice the threads per block (same arithmetic).  B = 1, N = 2^16: scalogram 26.6 ->
+// 22.5 us, gY spectra + second-order backward 76 -> 67, first-order backward 37 -> 26.5, g_x 39 -> 33;
+// with one block per SM the other blocks' latency hiding is not there to lose.
+inline bool few_blocks(const jtfs_plan* p, long long blocks) {
+  int n_sm = 148;
+  cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, p->device);
+  return blocks <= n_sm;
+}
 
 // x-hat by decimation: x_r[m] = x[r + D m] (D sub-sequences of length M), FFT each,
 // then x-hat[k] = sum_r exp(-2 pi i r k / N) X_r[k mod M].
-__global__ void __launch_bounds__(kFftThreads)
+template <int TH>
+__global__ void __launch_bounds__(TH)
 k_xfft_sub(DevPlan P, const float* __restrict__ x, float2* __restrict__ xsub) {
   pdl_enter();
   extern __shared__ float2 sm[];
@@ -30,6 +40,12 @@ k_xfft_sub(DevPlan P, const float* __restrict__ x, float2* __restrict__ xsub) {
   fft_dit_rows_r16<-1>(sm, P.logM, 1, twl_for(P, P.logM));
   float2* out = xsub + ((size_t)b * P.D + r) * P.M;
   for (int k = threadIdx.x; k < P.M; k += blockDim.x) out[k] = sm[fft_pos(k, P.logM)];
+}
+
+inline void launch_xfft_sub(const jtfs_plan* p, int B, const float* x, float2* xsub, cudaStream_t st) {
+  const bool few = few_blocks(p, (long long)p->dp.D * B);
+  launch_pdl(few ? k_xfft_sub<2 * kFftThreads> : k_xfft_sub<kFftThreads>, dim3(p->dp.D, B),
+             few ? 2 * kFftThreads : kFftThreads, (size_t)p->dp.M * 17 / 2, st, p->dp, x, xsub);
 }
 
 __global__ void k_xfft_combine(DevPlan P, const float2* __restrict__ xsub, float2* __restrict__ xh) {
