@@ -86,22 +86,28 @@ k_phi_fwd(DevPlan P, const float* __restrict__ s1, float* __restrict__ s2) {
   }
 }
 
+// Backward of one signal's paths over CW of the frames (grid: signals, frame groups).  The time
+// pooling's adjoint is taken before the lambda pooling's (they act on different axes), so all
+// that follows stays within a frame and frame groups are independent.  Bound by the serial chain
+// of one block, n_phi paths of 4 n1^2 CW multiply-adds: one block per signal took 333 us at
+// B = 33, n1 = 87, 32 frames, 8 paths.
 __global__ void __launch_bounds__(kPhiThreads)
-k_phi_bwd(DevPlan P, const float* __restrict__ s1, const float* __restrict__ gs2,
+k_phi_bwd(DevPlan P, int cw, const float* __restrict__ s1, const float* __restrict__ gs2,
           const float* __restrict__ gs1, float* __restrict__ gs1_out) {
   extern __shared__ float2 sm2[];
-  const int b = blockIdx.x;
-  const int n1 = P.n1, nt = P.n_t, nfm = P.N_fr - 1, cells = n1 * nt;
+  const int b = blockIdx.x, m0 = blockIdx.y * cw;
+  const int n1 = P.n1, nt = P.n_t, nfm = P.N_fr - 1, cells = n1 * cw;
   float2* h = sm2;                                    // [N_fr]
-  float* y = reinterpret_cast<float*>(h + P.N_fr);    // [n1][nt] S1
-  float* gy = y + cells;                              // [n1][nt] cotangent of S1
-  float* gr = gy + cells;                             // [n1][nt] g_|Z|, then Re gZ
-  float* gi = gr + cells;                             // [n1][nt] lambda-pooling adjoint, then Im gZ
+  float* y = reinterpret_cast<float*>(h + P.N_fr);    // [n1][cw] S1
+  float* gy = y + cells;                              // [n1][cw] cotangent of S1
+  float* gr = gy + cells;                             // [n1][cw] g_|Z|, then Re gZ
+  float* gi = gr + cells;                             // [n_lo][cw] time-pooling adjoint, then Im gZ
   float* wt = gi + cells;                             // [nt]
-  const float* src = s1 + (size_t)b * cells;
+  const size_t o = (size_t)b * n1 * nt + m0;
   for (int i = threadIdx.x; i < cells; i += blockDim.x) {
-    y[i] = src[i];
-    gy[i] = gs1 ? gs1[(size_t)b * cells + i] : 0.f;
+    const int lam = i / cw, m = i - lam * cw;
+    y[i] = s1[o + lam * nt + m];
+    gy[i] = gs1 ? gs1[o + lam * nt + m] : 0.f;
   }
   for (int i = threadIdx.x; i < nt; i += blockDim.x)
     wt[i] = (float)P.T * __ldg(&P.phiT[((long long)i * P.T) & (P.N - 1)]);
@@ -110,29 +116,29 @@ k_phi_bwd(DevPlan P, const float* __restrict__ s1, const float* __restrict__ gs2
     const float* g = gs2 + (size_t)b * P.s2_stride + ((size_t)P.n2 * P.C + q) * P.n_lo * nt;
     __syncthreads();   // the previous path is done with h, gr, gi
     for (int i = threadIdx.x; i < P.N_fr; i += blockDim.x) h[i] = P.h[(size_t)c * P.N_fr + i];
-    for (int i = threadIdx.x; i < cells; i += blockDim.x) {
-      const int lam = i / nt, t = i - lam * nt;
+    for (int i = threadIdx.x; i < P.n_lo * cw; i += blockDim.x) {
+      const int lo = i / cw, m = m0 + i - lo * cw;
       float acc = 0.f;
-      if (P.average_fr) {
-        for (int lo = 0; lo < P.n_lo; ++lo)
-          acc = fmaf(__ldg(&P.phiF[(lo * P.s_F - lam) & nfm]), g[lo * nt + t], acc);
-      } else {
-        acc = g[i];
-      }
+      for (int t = 0; t < nt; ++t) acc = fmaf(wt[(t - m) & (nt - 1)], __ldg(&g[lo * nt + t]), acc);
       gi[i] = acc;
     }
     __syncthreads();
     for (int i = threadIdx.x; i < cells; i += blockDim.x) {
-      const int lam = i / nt, m = i - lam * nt;
+      const int lam = i / cw, m = i - lam * cw;
       float acc = 0.f;
-      for (int t = 0; t < nt; ++t) acc = fmaf(wt[(t - m) & (nt - 1)], gi[lam * nt + t], acc);
+      if (P.average_fr) {
+        for (int lo = 0; lo < P.n_lo; ++lo)
+          acc = fmaf(__ldg(&P.phiF[(lo * P.s_F - lam) & nfm]), gi[lo * cw + m], acc);
+      } else {
+        acc = gi[i];
+      }
       gr[i] = acc;
     }
     __syncthreads();
     // gZ = g_|Z| Z / |Z| (0 where Z = 0), each cell in place
     for (int i = threadIdx.x; i < cells; i += blockDim.x) {
-      const int lam = i / nt, m = i - lam * nt;
-      const float2 z = lambda_conv(h, y, n1, nt, nfm, lam, m);
+      const int lam = i / cw, m = i - lam * cw;
+      const float2 z = lambda_conv(h, y, n1, cw, nfm, lam, m);
       const float a = sqrtf(z.x * z.x + z.y * z.y);
       const float s = a > 0.f ? gr[i] / a : 0.f;
       gr[i] = s * z.x;
@@ -141,18 +147,21 @@ k_phi_bwd(DevPlan P, const float* __restrict__ s1, const float* __restrict__ gs2
     __syncthreads();
     // g_S1[lam'][m] += sum_lam Re(conj(h[lam - lam']) gZ[lam][m])
     for (int i = threadIdx.x; i < cells; i += blockDim.x) {
-      const int lp = i / nt, m = i - lp * nt;
+      const int lp = i / cw, m = i - lp * cw;
       float acc = 0.f;
       for (int lam = 0; lam < n1; ++lam) {
         const float2 hv = h[(lam - lp) & nfm];
-        acc = fmaf(hv.x, gr[lam * nt + m], acc);
-        acc = fmaf(hv.y, gi[lam * nt + m], acc);
+        acc = fmaf(hv.x, gr[lam * cw + m], acc);
+        acc = fmaf(hv.y, gi[lam * cw + m], acc);
       }
       gy[i] += acc;
     }
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < cells; i += blockDim.x) gs1_out[(size_t)b * cells + i] = gy[i];
+  for (int i = threadIdx.x; i < cells; i += blockDim.x) {
+    const int lam = i / cw;
+    gs1_out[o + lam * nt + (i - lam * cw)] = gy[i];
+  }
 }
 
 // S1[lam][t] = sum_m s phi_T[(t T - m s) mod N] U1_lam[m] for the row of stride s.
@@ -231,7 +240,12 @@ jtfs_status launch_phi_backward(const jtfs_plan* p, int B, const float* s1, cons
   jtfs_status rc = cuda_check(cudaFuncSetAttribute(k_phi_bwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem), "attr");
   if (rc != JTFS_OK) return rc;
   StageScope sc(p, kStJointBwd, st, 1);
-  k_phi_bwd<<<B, kPhiThreads, smem, st>>>(p->dp, s1, gs2, gs1, gs1_out);
+  // frames per block: halved while the blocks do not fill the SMs twice and a block's cells still
+  // occupy its threads
+  int n_sm = 148, cw = p->n_t;
+  cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, p->device);
+  while (cw % 2 == 0 && p->n1 * cw / 2 >= kPhiThreads && (long long)B * (p->n_t / cw) < 2 * n_sm) cw /= 2;
+  k_phi_bwd<<<dim3(B, p->n_t / cw), kPhiThreads, smem, st>>>(p->dp, cw, s1, gs2, gs1, gs1_out);
   return cuda_check(cudaGetLastError(), "k_phi_bwd");
 }
 
