@@ -889,19 +889,19 @@ k_joint_fwd_tp(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
   uint8_t* sm = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   constexpr int BN = 64;
   constexpr int NP = PS * NT;                            // pooling N (frames of W_hi [, W_lo])
-  const int planes = args.passes == 3 ? 2 : 1;
+  constexpr int planes = PS;                             // W and Y planes
   const int S = args.stages, WS = args.wstages;
   constexpr uint32_t kAPlane = kBM * kBK * 2;            // 8 KB: 128 rows x 32 lambda', SW64
   constexpr uint32_t kYAtom = 4096;                      // 32 lambda' x 64 samples, SW128
   constexpr uint32_t kWHalf = NT * 64 * 2;               // one weight plane: NT frames x 64 samples
   const int max_kb = args.res_kb;
-  const uint32_t y_bytes = planes * 2 * kYAtom;          // per plane [Yr atom | Yi atom]
-  const uint32_t stage_bytes = RES ? y_bytes : planes * 2 * kAPlane + y_bytes;
+  constexpr uint32_t y_bytes = planes * 2 * kYAtom;          // per plane [Yr atom | Yi atom]
+  constexpr uint32_t stage_bytes = RES ? y_bytes : planes * 2 * kAPlane + y_bytes;
   uint8_t* sA = sm;
   uint8_t* sStage = sm + (RES ? planes * 2 * max_kb * kAPlane : 0);
   uint8_t* sWt = sStage + S * stage_bytes;               // WS slots of [W_hi plane][W_lo plane]
-  __shared__ uint64_t full_bar[8], empty_bar[8], wfull[kMaxWS], wempty[kMaxWS], tfull, tempty,
-      sfull, sfree, dfull, dfree, a_full, a_free, mma_done, pool_done, prod[2];
+  __shared__ uint64_t full_bar[8], empty_bar[8], wfull[kMaxWS], wempty[kMaxWS], tfull[2], tempty[2],
+      sfull, sfree, dfull, dfree, a_full, a_free, mma_done, pool_done;
   __shared__ uint32_t tmem_base;
   __shared__ volatile int abort_flag;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -916,8 +916,10 @@ k_joint_fwd_tp(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
       mbar_init(&wfull[s], 1);
       mbar_init(&wempty[s], 1);
     }
-    mbar_init(&tfull, 1);
-    mbar_init(&tempty, kEpiWarps);
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&tfull[i], 1);
+      mbar_init(&tempty[i], kEpiWarps);
+    }
     mbar_init(&sfull, kEpiWarps);
     mbar_init(&sfree, 1);
     mbar_init(&dfull, 1);
@@ -926,8 +928,6 @@ k_joint_fwd_tp(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
     mbar_init(&a_free, 1);
     mbar_init(&mma_done, 1);
     mbar_init(&pool_done, 1);
-    mbar_init(&prod[0], 1);
-    mbar_init(&prod[1], 1);
     fence_barrier_init();
   }
   if (warp == 1) {
@@ -974,7 +974,7 @@ k_joint_fwd_tp(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
           for (int pl = 0; pl < planes; ++pl)
             for (int part = 0; part < 2; ++part)
               for (int kb = 0; kb < nkb; ++kb)
-                tma_load_2d(sA + ((pl * 2 + part) * max_kb + kb) * kAPlane,
+                tma_load_2d(sA + (kb * planes * 2 + pl * 2 + part) * kAPlane,
                             &maps.w[pl * 2 + part], lm8 + kb * kBK, m0, &a_full);
           aph ^= 1;
         }
@@ -1019,7 +1019,7 @@ k_joint_fwd_tp(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
       const uint32_t id = instr_desc(kBM, 128, 1, 1, 0, 1, 0);
       constexpr int npair = PS == 2 ? 3 : 1;   // FP32-grade split, or one pass
       int stage = 0;
-      uint32_t phase = 0, tph = 0, aph = 0, par = 0;
+      uint32_t phase = 0, tph = 0, aph = 0;
       bool ok = true;
       for (int it = blockIdx.x; it < args.n_items && ok && !abort_flag; it += gridDim.x) {
         int b;
@@ -1033,44 +1033,68 @@ k_joint_fwd_tp(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
           aph ^= 1;
         }
         for (int j = 0; j < item.z && ok; ++j) {
-          // the first operand stage is there, as a rule, before the accumulator is free
-          if (!mbar_wait(&full_bar[stage], phase, wait_budget)) { fail(35); ok = false; break; }
-          if (!mbar_wait(&tempty, tph ^ 1, wait_budget)) { fail(34); ok = false; break; }
-          tph ^= 1;
-          const uint32_t t_a = tbase, t_b = tbase + 128;
-          for (int kb = 0; kb < nkb; ++kb) {
-            if (kb && !mbar_wait(&full_bar[stage], phase, wait_budget)) { fail(35); ok = false; break; }
-            tc_fence_after();
-            const uint32_t st = smem_u32(sStage + stage * stage_bytes);
+          const uint32_t t_ab[2] = {tbase, tbase + 128};   // [P1 | P3] = Wr [Yr | Yi], [P4 | P2] = Wi [Yr | Yi]
+          // halves h0 .. h1 of k-block kb (operand stage sg)
+          auto issue = [&](int kb, int sg, int h0, int h1) {
+            const uint32_t st = smem_u32(sStage + sg * stage_bytes);
             const uint32_t sb = RES ? st : st + planes * 2 * kAPlane;
-            const uint32_t sa = RES ? smem_u32(sA) + kb * kAPlane : st;
-            const uint32_t a_stride = RES ? max_kb * kAPlane : kAPlane;
+            const uint32_t sa = RES ? smem_u32(sA) + kb * planes * 2 * kAPlane : st;
             const int kss = min(2, nks - 2 * kb);
             const uint64_t dA = smem_desc(sa, 16, 512, kSw64);
             const uint64_t dB = smem_desc(sb, kYAtom, 1024, kSw128);
-            const uint32_t as4 = a_stride >> 4;
 #pragma unroll
             for (int ks = 0; ks < 2; ++ks) {
               if (ks < kss) {
 #pragma unroll
                 for (int q = 0; q < npair; ++q) {
                   const int pa = q == 2 ? 1 : 0, pb = q == 1 ? 1 : 0;
-                  const uint64_t ar = dA + (uint64_t)(pa * 2 * as4 + ks * 2);
-                  const uint64_t ai = ar + as4;
                   const uint64_t bd = dB + (uint64_t)(pb * 2 * (kYAtom >> 4) + ks * 128);
                   const uint32_t f = (kb | ks | q) ? 1u : 0u;
-                  mma_f16(t_a, ar, bd, id, f);    // [P1 | P3] = Wr [Yr | Yi]
-                  mma_f16(t_b, ai, bd, id, f);    // [P4 | P2] = Wi [Yr | Yi]
+#pragma unroll
+                  for (int hf = 0; hf < 2; ++hf)
+                    if (hf >= h0 && hf <= h1)
+                      mma_f16(t_ab[hf], dA + (uint64_t)((pa * 2 + hf) * (kAPlane >> 4) + ks * 2), bd, id, f);
                 }
               }
             }
-            mma_commit(&empty_bar[stage]);
-            if (++stage == S) { stage = 0; phase ^= 1; }
+          };
+          // the first operand stage is there, as a rule, before the accumulator is free
+          if (!mbar_wait(&full_bar[stage], phase, wait_budget)) { fail(35); ok = false; break; }
+          if (!mbar_wait(&tempty[0], tph ^ 1, wait_budget)) { fail(34); ok = false; break; }
+          if (nkb <= S) {
+            // one half after the other over all the k-blocks: the epilogue loads and frees a half
+            // while the other is computed
+            int sg = stage;
+            for (int kb = 0; kb < nkb; ++kb) {
+              if (kb && !mbar_wait(&full_bar[stage], phase, wait_budget)) { fail(35); ok = false; break; }
+              tc_fence_after();
+              issue(kb, stage, 0, 0);
+              if (++stage == S) { stage = 0; phase ^= 1; }
+            }
+            if (!ok) break;
+            mma_commit(&tfull[0]);
+            if (!mbar_wait(&tempty[1], tph ^ 1, wait_budget)) { fail(34); ok = false; break; }
+            tc_fence_after();
+            for (int kb = 0; kb < nkb; ++kb) {
+              issue(kb, sg, 1, 1);
+              mma_commit(&empty_bar[sg]);
+              if (++sg == S) sg = 0;
+            }
+          } else {
+            if (!mbar_wait(&tempty[1], tph ^ 1, wait_budget)) { fail(34); ok = false; break; }
+            for (int kb = 0; kb < nkb; ++kb) {
+              if (kb && !mbar_wait(&full_bar[stage], phase, wait_budget)) { fail(35); ok = false; break; }
+              tc_fence_after();
+              issue(kb, stage, 0, 1);
+              mma_commit(&empty_bar[stage]);
+              if (++stage == S) { stage = 0; phase ^= 1; }
+            }
+            if (!ok) break;
+            mma_commit(&tfull[0]);
           }
+          tph ^= 1;
           if (!ok) break;
-          mma_commit(&tfull);
-          mma_commit(&prod[par]);
-          par ^= 1;
+          mma_commit(&tfull[1]);
         }
         if (!ok) break;
         if (RES) mma_commit(&a_free);
@@ -1085,7 +1109,7 @@ k_joint_fwd_tp(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
       // samples] K-major with 128-byte rows; a K step is 16 samples
       const uint32_t idp = instr_desc(kBM, NP, 1, 1, 0, 0, 0);
       int ws = 0;
-      uint32_t sph = 0, wph = 0, dph = 0, tiles = 0;
+      uint32_t sph = 0, wph = 0, dph = 0;
       bool ok = true;
       for (int it = blockIdx.x; it < args.n_items && ok && !abort_flag; it += gridDim.x) {
         int b;
@@ -1096,13 +1120,6 @@ k_joint_fwd_tp(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
         for (int j = 0; j < item.z && ok; ++j) {
           if (!mbar_wait(&sfull, sph, wait_budget)) { fail(37); ok = false; break; }
           sph ^= 1;
-          // product t + 1 has completed (there is one unless this is the CTA's last tile): the
-          // pooling of tile t then runs while the epilogue loads that product, when the tensor
-          // pipe is idle.  Product t + 3, whose commit reuses this barrier, waits for the
-          // accumulator of tile t + 2 and so for this pooling: no phase can be missed.
-          ++tiles;
-          if ((j + 1 < item.z || it + (int)gridDim.x < args.n_items) &&
-              !mbar_wait(&prod[tiles & 1], (tiles >> 1) & 1, wait_budget)) { fail(42); ok = false; break; }
           if (!mbar_wait(&wfull[ws], wph, wait_budget)) { fail(38); ok = false; break; }
           tc_fence_after();
           const uint64_t dW = smem_desc(smem_u32(sWt + ws * PS * kWHalf), 16, 1024, kSw128);
@@ -1143,25 +1160,35 @@ k_joint_fwd_tp(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
       const int a = item.x, m0 = item.y;
       bool ok = !abort_flag;
       for (int j = 0; j < item.z && ok; ++j) {
-        if (!mbar_wait(&tfull, tph, wait_budget)) { fail(39); ok = false; break; }
-        tph ^= 1;
-        tc_fence_after();
         const uint32_t t_col = tbase + lane_off + cg * 16;
         uint32_t hv[2][2][4], lv[2][2][4];     // [h8][spin][4 bf16x2]
-        // the whole accumulator share (four products x 16 samples) is loaded before it is
-        // released, so the next tile's product waits for the loads alone
+        // each half of the accumulator share (two products x 16 samples) is loaded as soon as it is
+        // complete and released before any arithmetic
         uint32_t q1[2][8], q3[2][8], q4[2][8], q2[2][8];
+        if (!mbar_wait(&tfull[0], tph, wait_budget)) { fail(39); ok = false; break; }
+        tc_fence_after();
 #pragma unroll
         for (int h8 = 0; h8 < 2; ++h8) {
           tmem_ld8u(t_col + h8 * 8, q1[h8]);
           tmem_ld8u(t_col + h8 * 8 + 64, q3[h8]);
+        }
+        tmem_wait_ld();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&tempty[0]);
+        __syncwarp();
+        if (!mbar_wait(&tfull[1], tph, wait_budget)) { fail(39); ok = false; break; }
+        tph ^= 1;
+        tc_fence_after();
+#pragma unroll
+        for (int h8 = 0; h8 < 2; ++h8) {
           tmem_ld8u(t_col + h8 * 8 + 128, q4[h8]);
           tmem_ld8u(t_col + h8 * 8 + 192, q2[h8]);
         }
         tmem_wait_ld();
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(&tempty);
+        if (lane == 0) mbar_arrive(&tempty[1]);
         if (PS == 1) __syncwarp();             // the release before the arithmetic (1.6 %)
 #pragma unroll
         for (int h8 = 0; h8 < 2; ++h8) {
