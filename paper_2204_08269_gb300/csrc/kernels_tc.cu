@@ -868,15 +868,22 @@ k_joint_fwd_tc16(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
 // epilogue, at a quarter of the tcgen05 rate).  The epilogue stages |Z| (BF16 hi, lo for the
 // FP32-grade split) of both spins in tensor memory as an MMA A operand (row r in lane r, two
 // samples per 32-bit column: 32 columns per spin and plane), and a second issuing thread
-// (pooling tile t once product t + 1 has completed, when the tensor pipe is idle) accumulates D_spin[row][f] += |Z|[row][n] [W_hi | W_lo][f][n] over the item's tiles into TMEM
+// accumulates D_spin[row][f] += |Z|[row][n] [W_hi | W_lo][f][n] over the item's tiles into TMEM
 // (N = NT per weight plane: frames of W_hi, then of W_lo; both |Z| planes accumulate into the
 // same D, so D[f] + D[NT + f] = (Z_hi + Z_lo)(W_hi + W_lo)).  Staging |Z| in tensor memory
 // keeps its stores and the pooling MMAs' A reads off the shared memory, whose bandwidth the
 // product MMAs (8 KB per M = 128, N = 128, K = 16 step) already fill.  The TMEM holds one
-// 256-column product accumulator, the two pooling accumulators and the staged |Z|, so the
-// product of tile j + 1 starts once the epilogue has loaded tile j.  At an item's end warp
-// (quarter, cg) reads spin cg >> 1, frames [NT / 2 (cg & 1), +NT / 2) of its 32 rows and
-// writes them.
+// 256-column product accumulator, the two pooling accumulators and the staged |Z|.  The
+// accumulator changes hands by halves: [P1 | P3] over all the k-blocks, then [P4 | P2] (where the
+// operand stages hold a whole tile's k-blocks), so the epilogue loads and frees one half while the
+// tensor cores fill the other.  With one hand-off per tile the issuer waited 839 of a tile's 2744
+// cycles for it (FP32-grade; 916 of 1717 in BF16).  B = 64, N = 2^16, FP32-grade 4.62 -> 4.44 ms;
+// BF16, B = 256, N = 2^15, 5.88 -> 5.76 ms; Eq. 4 study, B = 64, 3.35 -> 3.20 ms.  Holding the
+// pooling back until the next product had completed, which paid with one hand-off, cost 3 % with
+// two.  What bounds it now is the epilogue (1400 to 1550 cycles of arithmetic per tile and 500 of
+// loads, stores and waits that its sixteen warps spend in step), then the tensor pipe (about
+// 1600).  At an item's end warp (quarter, cg) reads spin cg >> 1, frames [NT / 2 (cg & 1), +NT / 2)
+// of its 32 rows and writes them.
 constexpr int kTpThreads = 32 * 19;   // producer, product issuer, 16 epilogue warps, pooling issuer
 constexpr int kTpWarpPool = 18;
 
@@ -1330,7 +1337,8 @@ __global__ void __launch_bounds__(kPoolThreads)
 k_pool_lambda(DevPlan Pd, const float* __restrict__ P, const float* __restrict__ P2,
               long long part_stride, int part_samples, float* __restrict__ s2) {
   pdl_enter();
-  __shared__ float rows[kPoolRowsMax];
+  __shared__ __align__(16) float rows[kPoolRowsMax];
+  __shared__ float4 part4[kPoolThreads];
   __shared__ float phi[1024];
   const int a = blockIdx.x, b = blockIdx.y;
   const int c0 = Pd.C * blockIdx.z / gridDim.z, c1 = Pd.C * (blockIdx.z + 1) / gridDim.z;
@@ -1381,6 +1389,14 @@ k_pool_lambda(DevPlan Pd, const float* __restrict__ P, const float* __restrict__
     return;
   }
   for (int i = threadIdx.x; i < Pd.N_fr; i += blockDim.x) phi[i] = __ldg(&Pd.phiF[i]);
+  // A thread per (group of rows, output row, four frames) where those leave the block with two
+  // groups or more: four products per shared-memory pair of loads and a chain of n1 / G, against one
+  // thread per output that walks all n1 rows at two loads a product.  With the grouped k_g1, in one
+  // measurement: B = 5 in BF16 1128 -> 1076 us a step, B = 64 13.98 -> 13.87 ms.
+  const int nq = nout / 4, G = nt % 4 == 0 && nq <= kPoolThreads ? kPoolThreads / nq : 0;
+  const bool quads = G > 1;
+  const int g = quads ? threadIdx.x / nq : 0, lo = quads ? (threadIdx.x - g * nq) * 4 / nt : 0;
+  const int t0 = quads ? (threadIdx.x - g * nq) * 4 - lo * nt : 0;
   load(c0);
   for (int c = c0; c < c1; ++c) {
 #pragma unroll
@@ -1391,6 +1407,30 @@ k_pool_lambda(DevPlan Pd, const float* __restrict__ P, const float* __restrict__
     __syncthreads();
     if (c + 1 < c1) load(c + 1);
     float* out = out0 + (size_t)c * nout;
+    if (quads) {
+      // partial sums of rows g, g + G, ... for four frames of one output row
+      if (g < G) {
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        const int base = lo * Pd.s_F;
+#pragma unroll 4
+        for (int r = g; r < n1; r += G) {
+          const float f = phi[(base - r) & nfm];
+          const float4 x = *reinterpret_cast<const float4*>(&rows[r * nt + t0]);
+          v.x += f * x.x;
+          v.y += f * x.y;
+          v.z += f * x.z;
+          v.w += f * x.w;
+        }
+        part4[threadIdx.x] = v;
+      }
+      __syncthreads();
+      for (int i = threadIdx.x; i < nout; i += blockDim.x) {
+        float v = 0.f;
+        for (int q = 0; q < G; ++q) v += reinterpret_cast<const float*>(part4)[q * nout + i];
+        out[i] = v;
+      }
+      continue;   // (the next channel's barrier comes before part4 is written again)
+    }
     for (int i = threadIdx.x; i < nout; i += blockDim.x) {
       const int lo = i / nt, t = i - (i / nt) * nt;
       const int base = lo * Pd.s_F;

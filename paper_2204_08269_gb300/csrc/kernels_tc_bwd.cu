@@ -1581,8 +1581,8 @@ k_joint_bwd_pair(const __grid_constant__ TpMaps maps, TpArgs args, DevPlan P) {
 
 // G1[(b n2 + a) g1_rows + c n1 + lambda][t] = sum_lo phi_F[(lo s_F - lambda) mod N_fr] gS2[b,a,c,lo,t]
 // (or gS2 itself for Eq. 4), as BF16 (hi, and lo when g1lo is given), zero for t >= n_t.  One
-// block per (alpha, signal) walks the channels with phi_F and each channel's n_lo x n_t
-// cotangents in shared memory; every row adds its n_lo terms in increasing lo.  G1 rows are
+// block per (alpha, signal, share of the channels) walks groups of channels with phi_F and the
+// group's n_lo x n_t cotangents in shared memory; every row adds its n_lo terms in increasing lo.  G1 rows are
 // NT = 16 or 32 BF16 (32 or 64 bytes) from 16-byte aligned plane bases.
 constexpr int kG1Threads = 256;
 constexpr int kG1InMax = 4096;       // n_lo * n_t floats of one channel
@@ -1600,26 +1600,31 @@ k_g1(DevPlan Pd, const float* __restrict__ gs2, int NT, int g1_rows,
   const bool staged = nin <= kG1InMax && Pd.N_fr <= 1024;
   if (staged)
     for (int i = threadIdx.x; i < Pd.N_fr; i += blockDim.x) phi[i] = __ldg(&Pd.phiF[i]);
-  for (int c = c0; c < c1; ++c) {
-    const float* g = gs2 + (size_t)b * Pd.s2_stride + ((size_t)a * C + c) * Pd.n_lo * nt;
-    const size_t o0 = ((size_t)(b * Pd.n2 + a) * g1_rows + (size_t)c * n1) * NT;
+  // as many channels at a time as the staging holds (their cotangents are contiguous), so a group
+  // costs one round of loads and barriers
+  const int per = staged ? max(1, kG1InMax / nin) : c1 - c0;
+  const int ng = NT / 8;
+  for (int cs = c0; cs < c1; cs += per) {
+    const int nc = min(per, c1 - cs);
+    const float* g0 = gs2 + (size_t)b * Pd.s2_stride + ((size_t)a * C + cs) * Pd.n_lo * nt;
     if (staged) {
-      __syncthreads();   // the previous channel's reads are done
-      for (int i = threadIdx.x; i < nin; i += blockDim.x) gin[i] = g[i];
+      __syncthreads();   // the previous group's reads are done
+      for (int i = threadIdx.x; i < nc * nin; i += blockDim.x) gin[i] = g0[i];
       __syncthreads();
     }
     // eight frames per thread: one phi_F value serves eight outputs, and each plane takes one
     // 16-byte store (NT is 16 or 32, so a group never straddles rows)
-    const int ng = NT / 8;
-    for (int u = threadIdx.x; u < n1 * ng; u += blockDim.x) {
-      const int r = u / ng, t0 = (u - r * ng) * 8;
+    const size_t o0 = ((size_t)(b * Pd.n2 + a) * g1_rows + (size_t)cs * n1) * NT;
+    for (int u = threadIdx.x; u < nc * n1 * ng; u += blockDim.x) {
+      const int row = u / ng, t0 = (u - row * ng) * 8, c = row / n1, r = row - c * n1;
+      const float* g = (staged ? gin : g0) + c * nin;
       float s[8];
 #pragma unroll
       for (int k = 0; k < 8; ++k) s[k] = 0.f;
       if (Pd.average_fr) {
         for (int lo = 0; lo < Pd.n_lo; ++lo) {
           const float p = staged ? phi[(lo * Pd.s_F - r) & nfm] : __ldg(&Pd.phiF[(lo * Pd.s_F - r) & nfm]);
-          const float* gl = staged ? gin + lo * nt : g + lo * nt;
+          const float* gl = g + lo * nt;
 #pragma unroll
           for (int k = 0; k < 8; ++k)
             if (t0 + k < nt) s[k] += p * gl[t0 + k];
@@ -1627,7 +1632,7 @@ k_g1(DevPlan Pd, const float* __restrict__ gs2, int NT, int g1_rows,
       } else {
 #pragma unroll
         for (int k = 0; k < 8; ++k)
-          if (t0 + k < nt) s[k] = staged ? gin[r * nt + t0 + k] : g[r * nt + t0 + k];
+          if (t0 + k < nt) s[k] = g[r * nt + t0 + k];
       }
       uint32_t hw[4], lw[4];
 #pragma unroll
@@ -1638,7 +1643,7 @@ k_g1(DevPlan Pd, const float* __restrict__ gs2, int NT, int g1_rows,
         hw[k] = *reinterpret_cast<const uint32_t*>(&h);
         lw[k] = *reinterpret_cast<const uint32_t*>(&l);
       }
-      const size_t o = o0 + (size_t)r * NT + t0;
+      const size_t o = o0 + (size_t)row * NT + t0;
       *reinterpret_cast<uint4*>(g1 + o) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
       if (g1lo) *reinterpret_cast<uint4*>(g1lo + o) = make_uint4(lw[0], lw[1], lw[2], lw[3]);
     }
@@ -1742,7 +1747,8 @@ bool tcb_supported(const jtfs_plan* p) { return tc_nt(p->n_t) <= 64; }
 
 // CTAs per three-atom item: its chunks are the longest serial chain of the backward (201 us of the
 // 310 us contraction backward of one signal at N = 2^16), so a batch whose share per SM is less
-// than four such items splits them.
+// than four such items splits them (N = 2^16: one signal 263 -> 176 us with 8 parts, the five
+// signals of a BF16 batch 506 -> 462 us).
 int tcb_parts(const jtfs_plan* p, int B) {
   int n_sm = 148;
   cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, p->device);
