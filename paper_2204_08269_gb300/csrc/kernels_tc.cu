@@ -1213,8 +1213,8 @@ k_joint_fwd_tp(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
             const float2 su = __ffma2_rn(ru, ru, __fmul2_rn(iu, iu));
             const float2 sd = __ffma2_rn(rd, rd, __fmul2_rn(id, id));
             // one BF16 pass: subnormal |Z|^2 (|Z| < 1.1e-19) as 0, which halves the instructions of
-            // a root (6.70 -> 5.90 ms, B = 256, N = 2^15); the FP32-grade form keeps them, and
-            // measured slower without (5.22 against 4.64 ms, B = 64, N = 2^16)
+            // a root (6.70 -> 5.90 ms, B = 256, N = 2^15); the FP32-grade form keeps them (4.43
+            // against 4.21 ms, B = 64, N = 2^16)
             auto root = [](float v) { return PS == 1 ? sqrt_approx_ftz(v) : sqrt_approx(v); };
             const float2 mu = make_float2(root(su.x), root(su.y));
             const float2 md = make_float2(root(sd.x), root(sd.y));
