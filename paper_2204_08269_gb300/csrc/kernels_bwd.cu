@@ -3,9 +3,9 @@
 // backward recomputes x-hat, U1-hat, Y_alpha and Z, and the first-order coefficients z.
 //
 //   k_uh_from_u1       : U1-hat = FFT of every checkpointed U1 row
-//   k_joint_bwd_simt   : per (alpha, 32-column chunk, signal): for every channel c,
-//                        Z = W_c Y, g|Z| = adjoint of phi_T x phi_F pooling applied to g_S2,
-//                        gZ = g|Z| Z / |Z| (0 at Z = 0), gY += W_c^H gZ
+//   k_joint_bwd_simt   : per (alpha, 32- or 16-column chunk, signal): for every spin pair, then
+//                        phi_F: Z = W_c Y of both spins, g|Z| = adjoint of phi_T x phi_F pooling
+//                        applied to g_S2, gZ = g|Z| Z / |Z| (0 at Z = 0), gY += W_c^H gZ
 //   k_gy_spectra       : DFT of every gY row, in place (G rows of one rate per CTA)
 //   k_second_order_bwd : per (lambda', signal): sum over alpha of the adjoint of the
 //                        fold / psi_alpha product on those spectra, real part of the inverse
@@ -40,16 +40,17 @@ k_uh_from_u1(DevPlan P, const float* __restrict__ u1, float2* __restrict__ uh) {
 // Joint backward on CUDA cores (plain FP32 plans, and the rates past the tensor-core form's
 // lambda' range).  One CTA per (alpha, NC-column chunk, signal); it walks the spin pairs and then
 // the phi_F channel, whose filters W = Wr + i Wi serve both spins (the spin-down filter is the
-// conjugate of the spin-up one), so four real products per (row, lambda', column) give both Z:
-//   [P1 | P3] = Wr [Yr | Yi], [P4 | P2] = Wi [Yr | Yi],
-//   Z_up = (P1 - P2) + i (P3 + P4), Z_down = (P1 + P2) + i (P3 - P4),
-// and with S = gZ_up + gZ_down, T = (Im gZ_up - Im gZ_down) + i (Re gZ_down - Re gZ_up) the adjoint
+// conjugate of the spin-up one): Z_up = W Y and Z_down = conj(W) Y from one h per (row, lambda').
+// Each is summed product by product.  As P1 -/+ P2 of the real products Wr Y and Wi Y they take half
+// the FMAs, but a weak spin is then a difference of two sums of the strong one's size, and
+// gZ = g Z / |Z| weighs its cells like all others (a spin 54 times weaker, 151 rows: gradient
+// error 8.3e-7 so, 3.4e-6 as the difference).  B = 16, N = 2^17, n1 = 167, contraction backward:
+// 5.84 ms so, 5.11 as the difference.
+// With S = gZ_up + gZ_down, T = (Im gZ_up - Im gZ_down) + i (Re gZ_down - Re gZ_up) the adjoint
 // is gY += Wr^T S + Wi^T T (phi_F: Wi = 0, T unused).  Both products are bound by their FMAs: a
 // thread owns 8 consecutive rows x 4 columns, W is Toeplitz, so consecutive k shift an 8-entry
-// window of h by one and a step loads one h and four columns for 64 packed FMAs.  The gY
-// accumulators rest in shared memory while the Z product holds the registers.
-// B = 16, N = 2^17, the five lowest rates (167 lambda' rows): 6.00 -> 1.44 ms; the
-// earlier form took every spin by itself and loaded one h per four complex products.
+// window of h by one and a step loads one h and four columns for 128 packed FMAs (64 in the
+// adjoint).  The gY accumulators rest in shared memory while the Z product holds the registers.
 constexpr int kJR = 8;        // rows (or lambda') of a thread
 constexpr int kJC = 4;        // columns of a thread
 constexpr int kJT = 256;      // most threads: 256 / kJR row groups x 32 / kJC column groups
@@ -130,12 +131,12 @@ k_joint_bwd_simt(DevPlan P, const int2* __restrict__ items, const float2* __rest
       g1[i] = v;
     }
     __syncthreads();
-    // the products: pw = Wr Y, pi = Wi Y of rows r0 + i, columns col0 + CS j
-    float2 pw[kJR][kJC], pi[kJR][kJC];
+    // Z of both spins, rows r0 + i, columns col0 + CS j
+    float2 zu[kJR][kJC], zd[kJR][kJC];
 #pragma unroll
     for (int i = 0; i < kJR; ++i)
 #pragma unroll
-      for (int j = 0; j < kJC; ++j) pw[i][j] = pi[i][j] = make_float2(0.f, 0.f);
+      for (int j = 0; j < kJC; ++j) zu[i][j] = zd[i][j] = make_float2(0.f, 0.f);
     if (has_rows) {
       // row i's filter entry at step k is h[r0 + i - k - l0], in slot (i - k) mod 8
       float2 win[kJR];
@@ -146,16 +147,22 @@ k_joint_bwd_simt(DevPlan P, const int2* __restrict__ items, const float2* __rest
         for (int e = 0; e < kJR; ++e) {
           const int k = k0 + e;
           win[(kJR - e) & (kJR - 1)] = sh[max(r0 - k - l0, -Rp)];
-          float2 yv[kJC];
+          float2 yv[kJC], yi[kJC], yc[kJC];   // y, i y, -i y
 #pragma unroll
-          for (int j = 0; j < kJC; ++j) yv[j] = yt[k * NC + col0 + CS * j];
+          for (int j = 0; j < kJC; ++j) {
+            yv[j] = yt[k * NC + col0 + CS * j];
+            yi[j] = make_float2(-yv[j].y, yv[j].x);
+            yc[j] = make_float2(yv[j].y, -yv[j].x);
+          }
 #pragma unroll
           for (int i = 0; i < kJR; ++i) {
             const float2 w = win[(i - e + kJR) & (kJR - 1)];
 #pragma unroll
             for (int j = 0; j < kJC; ++j) {
-              pw[i][j] = __ffma2_rn(make_float2(w.x, w.x), yv[j], pw[i][j]);
-              pi[i][j] = __ffma2_rn(make_float2(w.y, w.y), yv[j], pi[i][j]);
+              zu[i][j] = __ffma2_rn(make_float2(w.x, w.x), yv[j], zu[i][j]);
+              zu[i][j] = __ffma2_rn(make_float2(w.y, w.y), yi[j], zu[i][j]);
+              zd[i][j] = __ffma2_rn(make_float2(w.x, w.x), yv[j], zd[i][j]);
+              zd[i][j] = __ffma2_rn(make_float2(w.y, w.y), yc[j], zd[i][j]);
             }
           }
         }
@@ -179,11 +186,10 @@ k_joint_bwd_simt(DevPlan P, const int2* __restrict__ items, const float2* __rest
         }
 #pragma unroll
         for (int j = 0; j < kJC; ++j) {
-          const float2 w = pw[i][j], q = pi[i][j];
-          const float2 zu = make_float2(w.x - q.y, w.y + q.x), zd = make_float2(w.x + q.y, w.y - q.x);
-          const float mu = sqrtf(zu.x * zu.x + zu.y * zu.y), md = sqrtf(zd.x * zd.x + zd.y * zd.y);
+          const float2 u = zu[i][j], d = zd[i][j];
+          const float mu = sqrtf(u.x * u.x + u.y * u.y), md = sqrtf(d.x * d.x + d.y * d.y);
           const float fu = mu > 0.f ? gu[j] / mu : 0.f, fd = md > 0.f ? gd[j] / md : 0.f;
-          const float2 zgu = make_float2(zu.x * fu, zu.y * fu), zgd = make_float2(zd.x * fd, zd.y * fd);
+          const float2 zgu = make_float2(u.x * fu, u.y * fu), zgd = make_float2(d.x * fd, d.y * fd);
           st[r * NC + col0 + CS * j] =
               pair ? make_float4(zgu.x + zgd.x, zgu.y + zgd.y, zgu.y - zgd.y, zgd.x - zgu.x)
                    : make_float4(zgu.x, zgu.y, 0.f, 0.f);
