@@ -44,16 +44,20 @@ k_uh_from_u1(DevPlan P, const float* __restrict__ u1, float2* __restrict__ uh) {
 // Each is summed product by product.  As P1 -/+ P2 of the real products Wr Y and Wi Y they take half
 // the FMAs, but a weak spin is then a difference of two sums of the strong one's size, and
 // gZ = g Z / |Z| weighs its cells like all others (a spin 54 times weaker, 151 rows: gradient
-// error 8.3e-7 so, 3.4e-6 as the difference).  B = 16, N = 2^17, n1 = 167, contraction backward:
-// 5.84 ms so, 5.11 as the difference.
+// error 8.3e-7 so, 3.4e-6 as the difference).
 // With S = gZ_up + gZ_down, T = (Im gZ_up - Im gZ_down) + i (Re gZ_down - Re gZ_up) the adjoint
 // is gY += Wr^T S + Wi^T T (phi_F: Wi = 0, T unused).  Both products are bound by their FMAs: a
-// thread owns 8 consecutive rows x 4 columns, W is Toeplitz, so consecutive k shift an 8-entry
-// window of h by one and a step loads one h and four columns for 128 packed FMAs (64 in the
+// thread owns 4 consecutive rows x 4 columns, W is Toeplitz, so consecutive k shift a 4-entry
+// window of h by one and a step loads one h and four columns for 64 packed FMAs (32 in the
 // adjoint).  The gY accumulators rest in shared memory while the Z product holds the registers.
-constexpr int kJR = 8;        // rows (or lambda') of a thread
+// Eight rows to a thread need fewer loads a product, but twice the registers and half the
+// threads, which short banks and many frames miss in the pooling adjoint.  Contraction backward in
+// plain FP32, 8 -> 4 rows (8 rows with Z as a difference in brackets): N = 2^12, n1 = 34, 64 frames,
+// B = 1 620 -> 265 us (572); N = 2^16, n1 = 151, B = 8 36.0 -> 22.8 ms (28.3); the step of B = 16,
+// N = 2^17, n1 = 167 with its five lowest rates here 5.84 -> 5.25 ms (5.11).
+constexpr int kJR = 4;        // rows (or lambda') of a thread
 constexpr int kJC = 4;        // columns of a thread
-constexpr int kJT = 256;      // most threads: 256 / kJR row groups x 32 / kJC column groups
+constexpr int kJT = 512;      // most threads: 32 columns fit the shared memory up to 223 rows, 16 to 256
 
 struct JointBwdLayout {       // float offsets in shared memory
   int rows, threads, y, st, gacc, h, g1, wt, total;
@@ -103,7 +107,10 @@ k_joint_bwd_simt(DevPlan P, const int2* __restrict__ items, const float2* __rest
     const int t = i / NC, n = n0 + i % NC;
     wt[i] = (n < A.L) ? __ldg(&P.phiT[(t * P.T - n * A.s) & (P.N - 1)]) * (float)A.s : 0.f;
   }
-  for (int i = 0; i < 2 * kJR * kJC; ++i) gacc[i * nthr + tid] = 0.f;
+  // the products' threads; the others only stage
+  const int na = lay.threads;
+  if (tid < na)
+    for (int i = 0; i < 2 * kJR * kJC; ++i) gacc[i * na + tid] = 0.f;
   // columns col0 + CS j: neighbouring lanes read neighbouring columns
   constexpr int CS = NC / kJC;
   const int col0 = tid % CS, r0 = tid / CS * kJR;
@@ -138,7 +145,7 @@ k_joint_bwd_simt(DevPlan P, const int2* __restrict__ items, const float2* __rest
 #pragma unroll
       for (int j = 0; j < kJC; ++j) zu[i][j] = zd[i][j] = make_float2(0.f, 0.f);
     if (has_rows) {
-      // row i's filter entry at step k is h[r0 + i - k - l0], in slot (i - k) mod 8
+      // row i's filter entry at step k is h[r0 + i - k - l0], in slot (i - k) mod kJR
       float2 win[kJR];
 #pragma unroll
       for (int i = 1; i < kJR; ++i) win[i] = sh[r0 + i - l0];
@@ -199,14 +206,14 @@ k_joint_bwd_simt(DevPlan P, const int2* __restrict__ items, const float2* __rest
     __syncthreads();
     if (has_k) {
       // gY[k][col] += sum_r Wr[r][k] S[r][col] + Wi[r][k] T[r][col], k = r0 + i: the filter entry
-      // h[r - k - l0] is in slot (r - i) mod 8
+      // h[r - k - l0] is in slot (r - i) mod kJR
       float2 acc[kJR][kJC];
 #pragma unroll
       for (int i = 0; i < kJR; ++i)
 #pragma unroll
         for (int j = 0; j < kJC; ++j)
-          acc[i][j] = make_float2(gacc[2 * (i * kJC + j) * nthr + tid],
-                                  gacc[(2 * (i * kJC + j) + 1) * nthr + tid]);
+          acc[i][j] = make_float2(gacc[2 * (i * kJC + j) * na + tid],
+                                  gacc[(2 * (i * kJC + j) + 1) * na + tid]);
       float2 win[kJR];
 #pragma unroll
       for (int i = 1; i < kJR; ++i) win[kJR - i] = sh[max(-(r0 + i) - l0, -Rp)];
@@ -231,8 +238,8 @@ k_joint_bwd_simt(DevPlan P, const int2* __restrict__ items, const float2* __rest
       for (int i = 0; i < kJR; ++i)
 #pragma unroll
         for (int j = 0; j < kJC; ++j) {
-          gacc[2 * (i * kJC + j) * nthr + tid] = acc[i][j].x;
-          gacc[(2 * (i * kJC + j) + 1) * nthr + tid] = acc[i][j].y;
+          gacc[2 * (i * kJC + j) * na + tid] = acc[i][j].x;
+          gacc[(2 * (i * kJC + j) + 1) * na + tid] = acc[i][j].y;
         }
     }
   }
@@ -244,8 +251,8 @@ k_joint_bwd_simt(DevPlan P, const int2* __restrict__ items, const float2* __rest
       for (int j = 0; j < kJC; ++j) {
         const int k = r0 + i, n = n0 + col0 + CS * j;
         if (k < K && n < A.L)
-          go[(size_t)k * A.L + n] = make_float2(gacc[2 * (i * kJC + j) * nthr + tid],
-                                                gacc[(2 * (i * kJC + j) + 1) * nthr + tid]);
+          go[(size_t)k * A.L + n] = make_float2(gacc[2 * (i * kJC + j) * na + tid],
+                                                gacc[(2 * (i * kJC + j) + 1) * na + tid]);
       }
   }
 }
@@ -648,14 +655,18 @@ jtfs_status set_attrs(const jtfs_plan* p) {
 }  // namespace
 
 // The CUDA-core joint backward over 32-column items: 32 columns at a time where the shared memory
-// holds them (every configuration but those with many rows and frames), else 16.
+// holds them (every configuration but those with many rows and frames), else 16.  Where the blocks
+// do not fill the SMs once they take at least 256 threads, whose surplus only stages: N = 512, n1 = 9,
+// 32 frames, B = 1 137 -> 107 us.
 static void launch_joint_bwd_simt(const jtfs_plan* p, int n_items, const int* items, int B,
                                   const float2* y, const float* gs2, float2* gy, cudaStream_t st) {
   const JointBwdLayout w = joint_bwd_layout(p->n1, p->n_t, 32);
   const bool wide = (size_t)w.total * 4 <= 227 * 1024;
   const JointBwdLayout l = wide ? w : joint_bwd_layout(p->n1, p->n_t, 16);
   auto* kernel = wide ? k_joint_bwd_simt<32> : k_joint_bwd_simt<16>;
-  launch_pdl(kernel, dim3((unsigned)n_items, B, wide ? 1 : 2), l.threads, (size_t)l.total * 4, st, p->dp, reinterpret_cast<const int2*>(items), y, gs2, gy);
+  const int threads = few_blocks(p, (long long)n_items * B) ? std::max(l.threads, 256) : l.threads;
+  launch_pdl(kernel, dim3((unsigned)n_items, B, wide ? 1 : 2), threads, (size_t)l.total * 4, st,
+             p->dp, reinterpret_cast<const int2*>(items), y, gs2, gy);
 }
 
 static void launch_second_order_bwd(const jtfs_plan* p, int B, const float2* gys, const float* gs1,
