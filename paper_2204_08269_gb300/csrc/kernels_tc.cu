@@ -1212,12 +1212,12 @@ k_joint_fwd_tp(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
             const float2 rd = __fadd2_rn(x1, x2), id = fsub2(x3, x4);
             const float2 su = __ffma2_rn(ru, ru, __fmul2_rn(iu, iu));
             const float2 sd = __ffma2_rn(rd, rd, __fmul2_rn(id, id));
-            // one BF16 pass: subnormal |Z|^2 (|Z| < 1.1e-19) as 0, which halves the instructions of
-            // a root (6.70 -> 5.90 ms, B = 256, N = 2^15); the FP32-grade form keeps them (4.43
-            // against 4.21 ms, B = 64, N = 2^16)
-            auto root = [](float v) { return PS == 1 ? sqrt_approx_ftz(v) : sqrt_approx(v); };
-            const float2 mu = make_float2(root(su.x), root(su.y));
-            const float2 md = make_float2(root(sd.x), root(sd.y));
+            // roots that keep subnormal |Z|^2 (|Z| < 1.1e-19): taken as 0 they would be half the
+            // instructions and quiet signals would lose their S2 (BF16, B = 256, N = 2^15: 6.62 ms
+            // so, 5.68 without; 6.31 where each row looks for such cells first, which the far
+            // tails of short wavelets have in any signal; FP32-grade, B = 64, N = 2^16: 4.43, 4.21)
+            const float2 mu = make_float2(sqrt_approx(su.x), sqrt_approx(su.y));
+            const float2 md = make_float2(sqrt_approx(sd.x), sqrt_approx(sd.y));
             __nv_bfloat162 hu = __floats2bfloat162_rn(mu.x, mu.y);
             __nv_bfloat162 hd = __floats2bfloat162_rn(md.x, md.y);
             hv[h8][0][i] = *reinterpret_cast<uint32_t*>(&hu);

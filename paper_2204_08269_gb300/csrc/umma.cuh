@@ -102,12 +102,6 @@ __device__ __forceinline__ float sqrt_approx(float x) {
   asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
   return r;
 }
-// The same with subnormal arguments taken as 0: no range fix-up around the instruction.
-__device__ __forceinline__ float sqrt_approx_ftz(float x) {
-  float r;
-  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
-}
 
 // Packed FP32 pairs (one instruction for two IEEE single operations, sm_100 and later): the
 // epilogues take their element pairs (k, k + 1) through these.  fsub2 is a - b as
