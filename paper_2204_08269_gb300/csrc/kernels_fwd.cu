@@ -41,7 +41,7 @@ constexpr int kS0Split = 8, kS0Threads = 256;
 
 __global__ void __cluster_dims__(kS0Split, 1, 1) __launch_bounds__(kS0Threads)
 k_s0(DevPlan P, const float* __restrict__ x, float* __restrict__ s0) {
-  pdl_trigger();
+  pdl_enter_early();
   __shared__ double red[kS0Threads / 32];
   __shared__ double parts[kS0Split];
   cg::cluster_group cl = cg::this_cluster();

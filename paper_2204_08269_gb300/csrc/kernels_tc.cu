@@ -170,10 +170,7 @@ k_joint_fwd_tc(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
   }
   __syncthreads();
   tc_fence_after();
-  // a launch that follows another form of the same stage is independent of it: it starts on the
-  // SMs the first one leaves and waits for it only at its end
-  if (!args.late) pdl_wait();
-  pdl_trigger();
+  pdl_enter_form(args.late);
   const uint32_t tbase = tmem_base;
   const uint32_t t_re = tbase, t_im = tbase + BN, t_pool = tbase + 2 * BN;
 
@@ -530,10 +527,7 @@ k_joint_fwd_tc16(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
   }
   __syncthreads();
   tc_fence_after();
-  // a launch that follows another form of the same stage is independent of it: it starts on the
-  // SMs the first one leaves and waits for it only at its end
-  if (!args.late) pdl_wait();
-  pdl_trigger();
+  pdl_enter_form(args.late);
   const uint32_t tbase = tmem_base;
 
   auto fail = [&](int code) {
@@ -943,10 +937,7 @@ k_joint_fwd_tp(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
   }
   __syncthreads();
   tc_fence_after();
-  // a launch that follows another form of the same stage is independent of it: it starts on the
-  // SMs the first one leaves and waits for it only at its end
-  if (!args.late) pdl_wait();
-  pdl_trigger();
+  pdl_enter_form(args.late);
   const uint32_t tbase = tmem_base;
   const uint32_t t_pool = tbase + 256;                   // [spin] NP columns each
   const uint32_t t_z = t_pool + 2 * NP;                  // [spin][plane] 32 columns of |Z|

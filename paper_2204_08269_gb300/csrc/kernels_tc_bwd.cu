@@ -113,8 +113,7 @@ k_joint_bwd_tc(const __grid_constant__ TbMaps maps, TbArgs args, DevPlan P) {
   }
   __syncthreads();
   tc_fence_after();
-  if (!args.late) pdl_wait();   // (a later form of the stage waits for the earlier one at its end)
-  pdl_trigger();
+  pdl_enter_form(args.late);
   const uint32_t tbase = tmem_base;
   auto fail = [&](int code) {
     if (!abort_flag) {
@@ -433,8 +432,7 @@ k_joint_bwd_tc3(const __grid_constant__ Tb3Maps maps, TbArgs args, DevPlan P) {
   }
   __syncthreads();
   tc_fence_after();
-  if (!args.late) pdl_wait();   // (a later form of the stage waits for the earlier one at its end)
-  pdl_trigger();
+  pdl_enter_form(args.late);
   const uint32_t tbase = tmem_base;
   auto fail = [&](int code) {
     if (!abort_flag) {
@@ -809,8 +807,7 @@ k_joint_bwd_fast(const __grid_constant__ TfMaps maps, TfArgs args, DevPlan P) {
   }
   __syncthreads();
   tc_fence_after();
-  if (!args.late) pdl_wait();   // (a later form of the stage waits for the earlier one at its end)
-  pdl_trigger();
+  pdl_enter_form(args.late);
   const uint32_t tbase = tmem_base;
   const uint32_t t_d2 = tbase + 6 * RC;                    // NAT x [Im 64 | Re 64]
   auto fail = [&](int code) {
@@ -1199,8 +1196,7 @@ k_joint_bwd_pair(const __grid_constant__ TpMaps maps, TpArgs args, DevPlan P) {
   }
   __syncthreads();
   tc_fence_after();
-  if (!args.late) pdl_wait();   // (a later form of the stage waits for the earlier one at its end)
-  pdl_trigger();
+  pdl_enter_form(args.late);
   const uint32_t tbase = tmem_base;
   // TMEM: 6 RC columns [P1 | P4] [P3 | P2] [g_up | g_dn] (2 RC apiece), then gY^T_re and gY^T_im
   // (64 NAT columns each), then S_re, S_im, T_re, T_im as the last product's A operand (RC pair

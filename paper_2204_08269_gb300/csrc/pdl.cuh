@@ -1,9 +1,22 @@
 // Programmatic dependent launch of the transform's kernel chain: a kernel is put on the SMs while
-// the last blocks of its predecessor still run, and blocks in pdl_enter until the predecessor has
-// completed and its writes are visible.  That hides the launch latency and the tail of every link
-// (a B = 1 step has 18 of them).  Every kernel launched through launch_pdl calls pdl_enter before
-// its first access to global memory that is not a constant of the plan; since each link waits for
-// the one before it, a kernel sees everything earlier in the stream.
+// the last blocks of its predecessor still run.  That hides the launch latency and the tail of every
+// link (a B = 1 step has 18 of them).  Every kernel launched through launch_pdl waits, on every way
+// out, until its predecessor has completed, so that its own completion means that everything before
+// it in the stream has completed.  They enter in one of three ways, before the first access to
+// global memory that is not a constant of the plan:
+//  - pdl_enter, nearly all: the dependents are let go, then the predecessor's completion is awaited.
+//  - pdl_enter_early: the kernel reads no result of its predecessor, only what was complete before
+//    that one let it go; it works beside the predecessor's tail and calls pdl_wait at its end.  k_s0
+//    (reads the call's input) and the contraction forms launched `late` (read Y, and G1 or the
+//    weights, as the form before them does).
+//  - pdl_enter_ordered: the wait comes before the dependents are let go.  A kernel after which an
+//    early one starts, directly or through kernels that let their dependents go at once, has to enter
+//    so: k_xfft_sub, the first kernel of every call, for k_s0 (the call's input is then complete), and
+//    the first form of a contraction stage for the later ones (Y and G1 are).
+// griddepcontrol.wait promises visibility to the grid that executes it.  An early kernel takes over
+// what the ordered one before it was promised: the writers are complete and their results in global
+// memory when that one triggers, the early grid starts after the trigger, and the fences on
+// both sides keep its reads from any older line of an L1.  TMA reads do not go through an L1.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -20,6 +33,20 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 __device__ __forceinline__ void pdl_enter() {
   pdl_trigger();
   pdl_wait();
+}
+__device__ __forceinline__ void pdl_enter_ordered() {
+  pdl_wait();
+  asm volatile("fence.acq_rel.gpu;" ::: "memory");
+  pdl_trigger();
+}
+__device__ __forceinline__ void pdl_enter_early() {   // pdl_wait at the kernel's end
+  asm volatile("fence.acq_rel.gpu;" ::: "memory");
+  pdl_trigger();
+}
+// A form of a contraction stage: the first one, or a later one (late), which is independent of it,
+// starts on the SMs that it leaves and calls pdl_wait at its end.
+__device__ __forceinline__ void pdl_enter_form(int late) {
+  if (late) pdl_enter_early(); else pdl_enter_ordered();
 }
 
 template <typename... Params, typename... Args>

@@ -30,10 +30,7 @@ inline bool few_blocks(const jtfs_plan* p, long long blocks) {
 template <int TH>
 __global__ void __launch_bounds__(TH)
 k_xfft_sub(DevPlan P, const float* __restrict__ x, float2* __restrict__ xsub) {
-  // wait, then trigger: every kernel after this one in the call starts with the call's inputs
-  // complete, also one that does not wait itself (k_s0)
-  pdl_wait();
-  pdl_trigger();
+  pdl_enter_ordered();   // every kernel after this one starts with the call's inputs complete
   extern __shared__ float2 sm[];
   const int r = blockIdx.x, b = blockIdx.y;
   const float* xb = x + (size_t)b * P.N;
