@@ -13,7 +13,7 @@
 // one spin is kept.
 //
 //   k_phi_fwd      : per (path, signal): the path from S1 into the tail of the signal's S2
-//   k_phi_bwd      : per signal: g_S1 + the adjoint of every path
+//   k_phi_bwd      : per (signal, frame group): g_S1 + the adjoint of every path
 //   k_s1_from_u1   : per (lambda, signal): S1 from the U1 checkpoint (Riemann sums in time),
 //                    for a backward call that did not run the forward
 //   k_pack_2d      : the 2-D layout, [out_rows][n_t] per signal: S0, S1 rows, S2 paths
@@ -25,6 +25,7 @@ namespace jtfs {
 namespace {
 
 constexpr int kPhiThreads = 256;
+constexpr size_t kPhiSmemMax = 227 * 1024;
 
 __device__ __forceinline__ int path_channel(const DevPlan& P, int q) {
   return (P.phi_psi && q < P.n_fr) ? q : 2 * P.n_fr;
@@ -205,16 +206,17 @@ __global__ void k_pack_2d(DevPlan P, float* s0, float* s1, float* s2, float* out
 size_t phi_fwd_smem(const jtfs_plan* p) {
   return (size_t)p->N_fr * 8 + (size_t)(2 * p->n1 * p->n_t + p->n_t) * 4;
 }
-size_t phi_bwd_smem(const jtfs_plan* p) {
-  return (size_t)p->N_fr * 8 + (size_t)(4 * p->n1 * p->n_t + p->n_t) * 4;
+// (a block of cw frames)
+size_t phi_bwd_smem(const jtfs_plan* p, int cw) {
+  return (size_t)p->N_fr * 8 + (size_t)(4 * p->n1 * cw + p->n_t) * 4;
 }
 
 }  // namespace
 
 bool phi_supported(const jtfs_plan* p) {
   // the phi_t paths' input is S1 itself only when phi_T's band is sampled at stride T
-  // (oversampling 0); one block holds the paths' whole [n1][n_t] planes
-  return p->cfg.oversampling == 0 && phi_bwd_smem(p) <= 227 * 1024;
+  // (oversampling 0); a block of a full batch's backward holds all the frames
+  return p->cfg.oversampling == 0 && phi_bwd_smem(p, p->n_t) <= kPhiSmemMax;
 }
 
 jtfs_status launch_phi_forward(const jtfs_plan* p, int B, const float* s1, float* s2,
@@ -236,8 +238,8 @@ jtfs_status launch_s1_from_u1(const jtfs_plan* p, int B, const float* u1, float*
 
 jtfs_status launch_phi_backward(const jtfs_plan* p, int B, const float* s1, const float* gs2,
                                 const float* gs1, float* gs1_out, cudaStream_t st) {
-  const size_t smem = phi_bwd_smem(p);
-  jtfs_status rc = cuda_check(cudaFuncSetAttribute(k_phi_bwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem), "attr");
+  // the attribute is the same for every call, the launch asks for what its frames take
+  jtfs_status rc = cuda_check(cudaFuncSetAttribute(k_phi_bwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPhiSmemMax), "attr");
   if (rc != JTFS_OK) return rc;
   StageScope sc(p, kStJointBwd, st, 1);
   // frames per block: halved while the blocks do not fill the SMs twice and a block's cells still
@@ -245,7 +247,7 @@ jtfs_status launch_phi_backward(const jtfs_plan* p, int B, const float* s1, cons
   int n_sm = 148, cw = p->n_t;
   cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, p->device);
   while (cw % 2 == 0 && p->n1 * cw / 2 >= kPhiThreads && (long long)B * (p->n_t / cw) < 2 * n_sm) cw /= 2;
-  k_phi_bwd<<<dim3(B, p->n_t / cw), kPhiThreads, smem, st>>>(p->dp, cw, s1, gs2, gs1, gs1_out);
+  k_phi_bwd<<<dim3(B, p->n_t / cw), kPhiThreads, phi_bwd_smem(p, cw), st>>>(p->dp, cw, s1, gs2, gs1, gs1_out);
   return cuda_check(cudaGetLastError(), "k_phi_bwd");
 }
 
