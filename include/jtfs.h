@@ -124,7 +124,10 @@ jtfs_status jtfs_workspace_bytes(const jtfs_plan* plan, int64_t B, int32_t with_
  * x [B, N] (device).  Writes s0, s1, s2 (device, sizes from
  * jtfs_plan_shapes).  With out_3d = 0, s0 receives the single [B, out_rows, n_t] output and
  * s1, s2 must be NULL.  u1_ckpt (device, [B, u1_len]) receives the first-order scalogram
- * checkpoint when not NULL; jtfs_backward needs it.  B = 0 is a no-op. */
+ * checkpoint when not NULL; jtfs_backward needs it.  B = 0 is a no-op.
+ * A signal's results do not depend on the other signals of the batch, but the last bits of its S2
+ * (and of g_x in jtfs_backward and the calls that include it) depend on B: small batches are cut
+ * into more pieces of work, which adds the same FP32 terms in another order. */
 jtfs_status jtfs_forward(const jtfs_plan* plan, const float* x, int64_t B, float* s0, float* s1,
                          float* s2, float* u1_ckpt, void* ws, size_t ws_bytes, void* stream);
 

@@ -41,8 +41,8 @@ k_uh_from_u1(DevPlan P, const float* __restrict__ u1, float2* __restrict__ uh) {
 // lambda' range).  One CTA per (alpha, NC-column chunk, signal); it walks the spin pairs and then
 // the phi_F channel, whose filters W = Wr + i Wi serve both spins (the spin-down filter is the
 // conjugate of the spin-up one): Z_up = W Y and Z_down = conj(W) Y from one h per (row, lambda').
-// Each is summed product by product.  As P1 -/+ P2 of the real products Wr Y and Wi Y they take half
-// the FMAs, but a weak spin is then a difference of two sums of the strong one's size, and
+// Each is summed product by product.  As P1 -/+ P2 of the real products Wr Y and Wi Y they take
+// half the FMAs, but a weak spin is then a difference of two sums of the strong one's size, and
 // gZ = g Z / |Z| weighs its cells like all others (a spin 54 times weaker, 151 rows: gradient
 // error 8.3e-7 so, 3.4e-6 as the difference).
 // With S = gZ_up + gZ_down, T = (Im gZ_up - Im gZ_down) + i (Re gZ_down - Re gZ_up) the adjoint
@@ -52,12 +52,12 @@ k_uh_from_u1(DevPlan P, const float* __restrict__ u1, float2* __restrict__ uh) {
 // adjoint).  The gY accumulators rest in shared memory while the Z product holds the registers.
 // Eight rows to a thread need fewer loads a product, but twice the registers and half the
 // threads, which short banks and many frames miss in the pooling adjoint.  Contraction backward in
-// plain FP32, 8 -> 4 rows (8 rows with Z as a difference in brackets): N = 2^12, n1 = 34, 64 frames,
-// B = 1 620 -> 265 us (572); N = 2^16, n1 = 151, B = 8 36.0 -> 22.8 ms (28.3); the step of B = 16,
-// N = 2^17, n1 = 167 with its five lowest rates here 5.84 -> 5.25 ms (5.11).
+// plain FP32, 8 -> 4 rows (8 rows with Z as a difference in brackets): N = 2^12, n1 = 34, B = 1,
+// 64 frames 620 -> 265 us (572); N = 2^16, n1 = 151, B = 8 36.0 -> 22.8 ms (28.3).  With the five
+// lowest rates alone here (B = 16, N = 2^17, n1 = 167) 5.84 -> 5.25 ms (5.11).
 constexpr int kJR = 4;        // rows (or lambda') of a thread
 constexpr int kJC = 4;        // columns of a thread
-constexpr int kJT = 512;      // most threads: 32 columns fit the shared memory up to 223 rows, 16 to 256
+constexpr int kJT = 512;      // most threads (32 columns fit the shared memory up to 220 rows, 448)
 
 struct JointBwdLayout {       // float offsets in shared memory
   int rows, threads, y, st, gacc, h, g1, wt, total;
@@ -656,8 +656,8 @@ jtfs_status set_attrs(const jtfs_plan* p) {
 
 // The CUDA-core joint backward over 32-column items: 32 columns at a time where the shared memory
 // holds them (every configuration but those with many rows and frames), else 16.  Where the blocks
-// do not fill the SMs once they take at least 256 threads, whose surplus only stages: N = 512, n1 = 9,
-// 32 frames, B = 1 137 -> 107 us.
+// do not fill the SMs once they take at least 256 threads, whose surplus only stages: N = 512,
+// n1 = 9, 32 frames, B = 1 137 -> 107 us.
 static void launch_joint_bwd_simt(const jtfs_plan* p, int n_items, const int* items, int B,
                                   const float2* y, const float* gs2, float2* gy, cudaStream_t st) {
   const JointBwdLayout w = joint_bwd_layout(p->n1, p->n_t, 32);
@@ -713,14 +713,18 @@ jtfs_status launch_backward(const jtfs_plan* p, const float* x, const float* u1,
     }
     {
       StageScope sc(p, kStUhFromU1, st, 1);
-      launch_pdl(k_uh_from_u1, dim3(p->n1, B), kFftThreads, (size_t)p->L1max * 17 / 2, st, d, u1, w.uh);
+      launch_pdl(k_uh_from_u1, dim3(p->n1, B), kFftThreads, (size_t)p->L1max * 17 / 2, st, d, u1,
+                 w.uh);
     }
   }
   const size_t n_items = p->items.size() / 2;
   if (gs2 && n_items > 0 && p->use_tcb) {
     if (!reuse_y) {
       StageScope sc(p, kStSecondOrder, st, 1);
-      launch_pdl(k_second_order_rows<1>, dim3((unsigned)(p->rowitems.size() / 4), B), p->row_threads, (size_t)p->rows_cap * 17 / 2, st, d, reinterpret_cast<const int4*>(p->d_rowitems), w.uh, nullptr, (__nv_bfloat16*)w.ybh, (__nv_bfloat16*)w.ybl, B);
+      launch_pdl(k_second_order_rows<1>, dim3((unsigned)(p->rowitems.size() / 4), B),
+                 p->row_threads, (size_t)p->rows_cap * 17 / 2, st, d,
+                 reinterpret_cast<const int4*>(p->d_rowitems), w.uh, nullptr, (__nv_bfloat16*)w.ybh,
+                 (__nv_bfloat16*)w.ybl, B);
     }
     StageScope sc(p, kStJointBwd, st, 0);   // the launcher counts its kernels
     jtfs_status r2 = launch_joint_bwd_tc(p, B, w.ybh, w.ybl, gs2, w.g1, w.gy, w.y, st);
@@ -728,7 +732,10 @@ jtfs_status launch_backward(const jtfs_plan* p, const float* x, const float* u1,
     if (!p->tcb_fb_items.empty()) {
       // rates beyond the tensor-core backward's lambda' capacity: FP32 Y rows of those rates
       // only, then the CUDA-core backward on them
-      launch_pdl(k_second_order_rows<0>, dim3((unsigned)(p->tcb_fb_rowitems.size() / 4), B), p->row_threads, (size_t)p->tcb_fb_cap * 17 / 2, st, d, reinterpret_cast<const int4*>(p->d_tcb_fb_rowitems), w.uh, w.y, nullptr, nullptr, B);
+      launch_pdl(k_second_order_rows<0>, dim3((unsigned)(p->tcb_fb_rowitems.size() / 4), B),
+                 p->row_threads, (size_t)p->tcb_fb_cap * 17 / 2, st, d,
+                 reinterpret_cast<const int4*>(p->d_tcb_fb_rowitems), w.uh, w.y, nullptr, nullptr,
+                 B);
       launch_joint_bwd_simt(p, (int)(p->tcb_fb_items.size() / 2), p->d_tcb_fb_items, B, w.y, gs2,
                             w.gy, st);
       p->prof.launches += 2;
@@ -736,7 +743,9 @@ jtfs_status launch_backward(const jtfs_plan* p, const float* x, const float* u1,
   } else if (gs2 && n_items > 0) {
     {
       StageScope sc(p, kStSecondOrder, st, 1);
-      launch_pdl(k_second_order_rows<0>, dim3((unsigned)(p->rowitems.size() / 4), B), p->row_threads, (size_t)p->rows_cap * 17 / 2, st, d, reinterpret_cast<const int4*>(p->d_rowitems), w.uh, w.y, nullptr, nullptr, B);
+      launch_pdl(k_second_order_rows<0>, dim3((unsigned)(p->rowitems.size() / 4), B),
+                 p->row_threads, (size_t)p->rows_cap * 17 / 2, st, d,
+                 reinterpret_cast<const int4*>(p->d_rowitems), w.uh, w.y, nullptr, nullptr, B);
     }
     StageScope sc(p, kStJointBwd, st, 1);
     launch_joint_bwd_simt(p, (int)n_items, p->d_items, B, w.y, gs2, w.gy, st);
@@ -748,7 +757,9 @@ jtfs_status launch_backward(const jtfs_plan* p, const float* x, const float* u1,
   {
     StageScope sc(p, kStSecondOrderBwd, st, 2);
     if (!p->rowitems.empty())
-      launch_pdl(k_gy_spectra, dim3((unsigned)(p->rowitems.size() / 4), B), p->row_threads, (size_t)p->rows_cap * 17 / 2, st, d, reinterpret_cast<const int4*>(p->d_rowitems), w.gy, gp);
+      launch_pdl(k_gy_spectra, dim3((unsigned)(p->rowitems.size() / 4), B), p->row_threads,
+                 (size_t)p->rows_cap * 17 / 2, st, d, reinterpret_cast<const int4*>(p->d_rowitems),
+                 w.gy, gp);
     launch_second_order_bwd(p, B, w.gy, gs1, w.gu1, st);
   }
   {
@@ -778,21 +789,26 @@ jtfs_status launch_scat1d_backward(const jtfs_plan* p, const float* x, const flo
   }
   {
     StageScope sc(p, kStUhFromU1, st, 1);
-    launch_pdl(k_uh_from_u1, dim3(p->n1, B), kFftThreads, (size_t)p->L1max * 17 / 2, st, d, u1, w.uh);
+    launch_pdl(k_uh_from_u1, dim3(p->n1, B), kFftThreads, (size_t)p->L1max * 17 / 2, st, d, u1,
+               w.uh);
   }
   if (gs2t && !p->rowitems.empty()) {
     StageScope sc(p, kStJointBwd, st, 1);
     auto* kernel = p->n_t >= 8 ? k_scat1d_bwd_rows<8>
                    : p->n_t == 4 ? k_scat1d_bwd_rows<4>
                    : p->n_t == 2 ? k_scat1d_bwd_rows<2> : k_scat1d_bwd_rows<1>;
-    launch_pdl(kernel, dim3((unsigned)(p->rowitems.size() / 4), B), p->row_threads, (size_t)p->rows_cap * 17 / 2, st, d, reinterpret_cast<const int4*>(p->d_rowitems), w.uh, gs2t, w.gy);
+    launch_pdl(kernel, dim3((unsigned)(p->rowitems.size() / 4), B), p->row_threads,
+               (size_t)p->rows_cap * 17 / 2, st, d, reinterpret_cast<const int4*>(p->d_rowitems),
+               w.uh, gs2t, w.gy);
   } else if (p->y_len > 0) {
     cudaMemsetAsync(w.gy, 0, (size_t)B * p->y_len * sizeof(float2), st);
   }
   {
     StageScope sc(p, kStSecondOrderBwd, st, 2);
     if (!p->rowitems.empty())
-      launch_pdl(k_gy_spectra, dim3((unsigned)(p->rowitems.size() / 4), B), p->row_threads, (size_t)p->rows_cap * 17 / 2, st, d, reinterpret_cast<const int4*>(p->d_rowitems), w.gy, GyParts{nullptr, 0, 0, 0, 0, 1});
+      launch_pdl(k_gy_spectra, dim3((unsigned)(p->rowitems.size() / 4), B), p->row_threads,
+                 (size_t)p->rows_cap * 17 / 2, st, d, reinterpret_cast<const int4*>(p->d_rowitems),
+                 w.gy, GyParts{nullptr, 0, 0, 0, 0, 1});
     launch_second_order_bwd(p, B, w.gy, gs1, w.gu1, st);
   }
   {

@@ -498,9 +498,12 @@ jtfs_status autotune_rows(jtfs_plan* p, int B, const Workspace& w, cudaStream_t 
         const dim3 grid((unsigned)(items.size() / 4), B);
         const size_t smem = (size_t)caps[ci] * 17 / 2;   // padded one per 16
         if (p->use_tc)
-          launch_pdl(k_second_order_rows<1>, grid, threads, smem, st, d, reinterpret_cast<const int4*>(d_items), w.uh, nullptr, (__nv_bfloat16*)w.ybh, (__nv_bfloat16*)w.ybl, B);
+          launch_pdl(k_second_order_rows<1>, grid, threads, smem, st, d,
+                     reinterpret_cast<const int4*>(d_items), w.uh, nullptr, (__nv_bfloat16*)w.ybh,
+                     (__nv_bfloat16*)w.ybl, B);
         else
-          launch_pdl(k_second_order_rows<0>, grid, threads, smem, st, d, reinterpret_cast<const int4*>(d_items), w.uh, w.y, nullptr, nullptr, B);
+          launch_pdl(k_second_order_rows<0>, grid, threads, smem, st, d,
+                     reinterpret_cast<const int4*>(d_items), w.uh, w.y, nullptr, nullptr, B);
       };
       launch();
       cudaEventRecord(e0, st);
@@ -567,7 +570,9 @@ jtfs_status launch_scat1d_forward(const jtfs_plan* p, const float* x, int B, flo
     auto* kernel = p->n_t >= 8 ? k_scat1d_rows<8>
                    : p->n_t == 4 ? k_scat1d_rows<4>
                    : p->n_t == 2 ? k_scat1d_rows<2> : k_scat1d_rows<1>;
-    launch_pdl(kernel, dim3((unsigned)(p->rowitems.size() / 4), B), p->row_threads, (size_t)p->rows_cap * 17 / 2, st, d, reinterpret_cast<const int4*>(p->d_rowitems), w.uh, s2t);
+    launch_pdl(kernel, dim3((unsigned)(p->rowitems.size() / 4), B), p->row_threads,
+               (size_t)p->rows_cap * 17 / 2, st, d, reinterpret_cast<const int4*>(p->d_rowitems),
+               w.uh, s2t);
   }
   return cuda_check(cudaGetLastError(), "time scattering forward");
 }
@@ -598,14 +603,17 @@ jtfs_status launch_forward(const jtfs_plan* p, const float* x, int B, float* s0,
     // TF32 operands: Y as FP32 planes (in the complex FP32 buffer, same size)
     if (!p->pairs.empty()) {
       StageScope sc(p, kStSecondOrder, st, 1);
-      launch_pdl(k_second_order_rows<2>, dim3((unsigned)(p->rowitems.size() / 4), B), p->row_threads, (size_t)p->rows_cap * 17 / 2, st, d, reinterpret_cast<const int4*>(p->d_rowitems), w.uh, w.y, nullptr, nullptr, B);
+      launch_pdl(k_second_order_rows<2>, dim3((unsigned)(p->rowitems.size() / 4), B),
+                 p->row_threads, (size_t)p->rows_cap * 17 / 2, st, d,
+                 reinterpret_cast<const int4*>(p->d_rowitems), w.uh, w.y, nullptr, nullptr, B);
     }
     {
       StageScope sc(p, kStSecondOrder, st, 0);
       for (int a = 0; a < p->n2; ++a) {
         const Rate2& A = p->rates2[a];
         if (A.s == 0 || A.kt == 0) continue;
-        launch_pdl(k_transpose_yt, dim3((A.L + 31) / 32, (A.kt + 31) / 32, 2 * B), dim3(32, 8), 0, st, d, a, reinterpret_cast<const float*>(w.y), w.yt, B);
+        launch_pdl(k_transpose_yt, dim3((A.L + 31) / 32, (A.kt + 31) / 32, 2 * B), dim3(32, 8), 0,
+                   st, d, a, reinterpret_cast<const float*>(w.y), w.yt, B);
         ++p->prof.launches;
       }
     }
@@ -615,7 +623,10 @@ jtfs_status launch_forward(const jtfs_plan* p, const float* x, int B, float* s0,
   } else if (p->use_tc) {
     if (!p->pairs.empty()) {
       StageScope sc(p, kStSecondOrder, st, 1);
-      launch_pdl(k_second_order_rows<1>, dim3((unsigned)(p->rowitems.size() / 4), B), p->row_threads, (size_t)p->rows_cap * 17 / 2, st, d, reinterpret_cast<const int4*>(p->d_rowitems), w.uh, nullptr, (__nv_bfloat16*)w.ybh, (__nv_bfloat16*)w.ybl, B);
+      launch_pdl(k_second_order_rows<1>, dim3((unsigned)(p->rowitems.size() / 4), B),
+                 p->row_threads, (size_t)p->rows_cap * 17 / 2, st, d,
+                 reinterpret_cast<const int4*>(p->d_rowitems), w.uh, nullptr, (__nv_bfloat16*)w.ybh,
+                 (__nv_bfloat16*)w.ybl, B);
     }
     StageScope sc(p, kStJointFwd, st, 0);   // the launcher counts its kernels
     // (the FP32 Y buffer is free here)
@@ -624,7 +635,9 @@ jtfs_status launch_forward(const jtfs_plan* p, const float* x, int B, float* s0,
   } else {
     if (!p->pairs.empty()) {
       StageScope sc(p, kStSecondOrder, st, 1);
-      launch_pdl(k_second_order_rows<0>, dim3((unsigned)(p->rowitems.size() / 4), B), p->row_threads, (size_t)p->rows_cap * 17 / 2, st, d, reinterpret_cast<const int4*>(p->d_rowitems), w.uh, w.y, nullptr, nullptr, B);
+      launch_pdl(k_second_order_rows<0>, dim3((unsigned)(p->rowitems.size() / 4), B),
+                 p->row_threads, (size_t)p->rows_cap * 17 / 2, st, d,
+                 reinterpret_cast<const int4*>(p->d_rowitems), w.uh, w.y, nullptr, nullptr, B);
     }
     StageScope sc(p, kStJointFwd, st, 1);
     launch_pdl(k_joint_fwd_simt, dim3(p->C, p->n2, B), kJT, joint_fwd_smem(p), st, d, w.y, s2);

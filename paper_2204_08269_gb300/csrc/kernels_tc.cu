@@ -539,7 +539,7 @@ k_joint_fwd_tc16(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
-    if (lane == 0) {
+    if (lane == 0) {   // (1 % faster here than elect_one)
       int stage = 0, ws = 0;
       uint32_t phase = 0, wph = 0, aph = 0;
       uint32_t armed = 0, armed_par = 0, armed_w = 0, armed_w_par = 0;
@@ -609,7 +609,7 @@ k_joint_fwd_tc16(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
+    if (lane == 0) {   // (1 % faster here than elect_one)
       constexpr uint32_t kFmt = TF ? 2 : 1;
       const uint32_t id_pos = instr_desc(kBM, BN, kFmt, kFmt, 0, TF ? 0 : 1, 0);
       const uint32_t id_neg = instr_desc(kBM, BN, kFmt, kFmt, 0, TF ? 0 : 1, 1);
@@ -1318,9 +1318,12 @@ k_joint_fwd_tp(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
 
 // phi_F pooling along lambda of the time-pooled rows: S2[b, a, c, lo, t] =
 // sum_lambda phi_F[(lo s_F - lambda) mod N_fr] P[b, a, c, lambda, t] (or P itself for Eq. 4).
-// One block per (alpha, signal) walks the channels: each channel's n1 x n_t rows (contiguous
-// in P) are staged in shared memory, the next channel's already in flight in registers, and
-// every output adds its n1 terms in increasing lambda.
+// A row of P is the sum of the rate's parts, added in their order.  One block per (alpha, signal,
+// share of the channels: channel_split) walks its channels: each channel's n1 x n_t rows
+// (contiguous in P) are staged in shared memory, the next channel's already in flight in
+// registers.  With G groups of threads (quads, below) an output is the sum of G partials, group g's
+// over the rows g, g + G, ... in increasing lambda, added in increasing g; without, or for rows
+// that are not staged, its n1 terms are added in increasing lambda.
 constexpr int kPoolThreads = 256;
 constexpr int kPoolRowsMax = 8192;   // n1 * n_t floats staged per channel
 
@@ -1697,9 +1700,12 @@ jtfs_status build_tc_tables(jtfs_plan* p) {
   // The longest rates walked whole (level 0), or in 2, 4 or 8 parts of equal numbers of tiles,
   // whose pooled rows k_pool_lambda adds: a batch too small to fill the SMs with whole rates takes
   // the first level whose longest item is at most 0.3 of an SM's share of the work (with no more
-  // than 0.3 the last items end close together; more parts cost a W load and a row write each).
-  // N = 2^16, whole rates -> parts: one signal, FP32-grade, contraction forward 272 -> 127 us (8
-  // parts); five, BF16, 732 -> 324 us (4); one signal of 2^12 in the 64-frame form 59 -> 36 us (2).
+  // than 0.3 the last items end close together; more parts cost a W load and a row write each), or
+  // the last one whose rows find room: parts past the first write theirs to the FP32 Y buffer, which
+  // holds 2 y_len floats a signal.  That is six sets of rows at N = 2^16 with 16 frames (so 4 parts,
+  // although one signal would take 8) and one where the frames are many (2^13 with 32 frames, 2^12
+  // with 64).  N = 2^16, whole rates -> 4 parts: one signal, FP32-grade, contraction forward 272 ->
+  // 127 us; five, BF16, 732 -> 324 us; one signal of 2^12 in the 64-frame form, 2 parts, 59 -> 36.
   p->tc_items.clear();
   p->tc_levels.clear();
   for (int parts = 1; parts <= 8 && (parts == 1 || max_tiles >= parts); parts *= 2) {

@@ -1,18 +1,18 @@
 // Programmatic dependent launch of the transform's kernel chain: a kernel is put on the SMs while
-// the last blocks of its predecessor still run.  That hides the launch latency and the tail of every
-// link (a B = 1 step has 18 of them).  Every kernel launched through launch_pdl waits, on every way
-// out, until its predecessor has completed, so that its own completion means that everything before
-// it in the stream has completed.  They enter in one of three ways, before the first access to
-// global memory that is not a constant of the plan:
-//  - pdl_enter, nearly all: the dependents are let go, then the predecessor's completion is awaited.
+// the last blocks of its predecessor still run.  That hides the launch latency and the tail of
+// every link (a B = 1 step has 18 of them).  Every kernel launched through launch_pdl waits, on
+// every way out, until its predecessor has completed, so that its own completion means that
+// everything before it in the stream has completed.  They enter in one of three ways, before the
+// first access to global memory that is not a constant of the plan:
+//  - pdl_enter, nearly all: the dependents are let go, then the predecessor's end is awaited.
 //  - pdl_enter_early: the kernel reads no result of its predecessor, only what was complete before
-//    that one let it go; it works beside the predecessor's tail and calls pdl_wait at its end.  k_s0
-//    (reads the call's input) and the contraction forms launched `late` (read Y, and G1 or the
+//    that one let it go; it works beside the predecessor's tail and calls pdl_wait at its end.
+//    k_s0 (reads the call's input) and the contraction forms launched `late` (read Y, and G1 or the
 //    weights, as the form before them does).
 //  - pdl_enter_ordered: the wait comes before the dependents are let go.  A kernel after which an
-//    early one starts, directly or through kernels that let their dependents go at once, has to enter
-//    so: k_xfft_sub, the first kernel of every call, for k_s0 (the call's input is then complete), and
-//    the first form of a contraction stage for the later ones (Y and G1 are).
+//    early one starts, directly or through kernels that let their dependents go at once, has to
+//    enter so: k_xfft_sub, the first kernel of every call, for k_s0 (the call's input is then
+//    complete), and the first form of a contraction stage for the later ones (Y and G1 are).
 // griddepcontrol.wait promises visibility to the grid that executes it.  An early kernel takes over
 // what the ordered one before it was promised: the writers are complete and their results in global
 // memory when that one triggers, the early grid starts after the trigger, and the fences on

@@ -18,7 +18,8 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
 // uniform registers, and only behind elect.sync does the compiler know that one lane is active and
 // move them there without a loop over the active lanes.  Against `lane == 0` (B = 64, N = 2^16,
 // FP32-grade) the issuing threads' cost per MMA fell enough to take the contraction forward from
-// 5.73 to 4.89 ms and the backward from 8.35 to 7.60 ms.
+// 5.73 to 4.89 ms and the backward from 8.35 to 7.60 ms.  One kernel keeps the lane index: the
+// TF32 forward (k_joint_fwd_tc16) measured 1 % slower with this.
 __device__ __forceinline__ bool elect_one() {
   uint32_t ok;
   asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}\n"

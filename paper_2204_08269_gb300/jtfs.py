@@ -262,7 +262,9 @@ class JTFSPlan:
 
     def forward(self, x, keep_checkpoint=True):
         """S0 [B, n_t], S1 [B, n1, n_t], S2 (see Shapes.s2) and the U1 checkpoint; in the 2-D
-        layout (out_3d=False) the single [B, out_rows, n_t] output and None, None."""
+        layout (out_3d=False) the single [B, out_rows, n_t] output and None, None.  The last
+        bits of S2 (and of a backward's g_x) depend on B: small batches are cut into more pieces
+        of work, whose sums are in another order."""
         self._check_x(x)
         B = x.shape[0]
         sh = self.shapes
