@@ -1187,7 +1187,6 @@ k_joint_fwd_tp(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(&tempty[1]);
-        if (PS == 1) __syncwarp();             // the release before the arithmetic (1.6 %)
 #pragma unroll
         for (int h8 = 0; h8 < 2; ++h8) {
           const uint32_t* p1 = q1[h8];
