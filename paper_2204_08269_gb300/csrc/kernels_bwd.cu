@@ -665,8 +665,8 @@ static void launch_joint_bwd_simt(const jtfs_plan* p, int n_items, const int* it
   const JointBwdLayout l = wide ? w : joint_bwd_layout(p->n1, p->n_t, 16);
   auto* kernel = wide ? k_joint_bwd_simt<32> : k_joint_bwd_simt<16>;
   const int threads = few_blocks(p, (long long)n_items * B) ? std::max(l.threads, 256) : l.threads;
-  launch_pdl(kernel, dim3((unsigned)n_items, B, wide ? 1 : 2), threads, (size_t)l.total * 4, st,
-             p->dp, reinterpret_cast<const int2*>(items), y, gs2, gy);
+  launch_spread(kernel, dim3((unsigned)n_items, B, wide ? 1 : 2), threads, (size_t)l.total * 4, st,
+                p->dp, reinterpret_cast<const int2*>(items), y, gs2, gy);
 }
 
 static void launch_second_order_bwd(const jtfs_plan* p, int B, const float2* gys, const float* gs1,

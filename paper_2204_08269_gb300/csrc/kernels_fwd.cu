@@ -640,7 +640,7 @@ jtfs_status launch_forward(const jtfs_plan* p, const float* x, int B, float* s0,
                  reinterpret_cast<const int4*>(p->d_rowitems), w.uh, w.y, nullptr, nullptr, B);
     }
     StageScope sc(p, kStJointFwd, st, 1);
-    launch_pdl(k_joint_fwd_simt, dim3(p->C, p->n2, B), kJT, joint_fwd_smem(p), st, d, w.y, s2);
+    launch_spread(k_joint_fwd_simt, dim3(p->C, p->n2, B), kJT, joint_fwd_smem(p), st, d, w.y, s2);
   }
   return cuda_check(cudaGetLastError(), "forward launch");
 }

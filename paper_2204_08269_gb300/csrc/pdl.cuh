@@ -50,8 +50,8 @@ __device__ __forceinline__ void pdl_enter_form(int late) {
 }
 
 template <typename... Params, typename... Args>
-inline void launch_pdl(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem,
-                       cudaStream_t st, Args&&... args) {
+inline void launch_chain(bool early, void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem,
+                         cudaStream_t st, Args&&... args) {
   cudaLaunchAttribute attr = {};
   attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr.val.programmaticStreamSerializationAllowed = 1;
@@ -61,8 +61,24 @@ inline void launch_pdl(void (*kernel)(Params...), dim3 grid, dim3 block, size_t 
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cfg.attrs = &attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = early ? 1 : 0;
   cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);   // errors: cudaGetLastError
+}
+
+template <typename... Params, typename... Args>
+inline void launch_pdl(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem,
+                       cudaStream_t st, Args&&... args) {
+  launch_chain(true, kernel, grid, block, smem, st, std::forward<Args>(args)...);
+}
+
+// The same, not before the predecessor has completed: for kernels of few and long blocks that fit
+// an SM several at a time.  Put on the SMs early they gather on those that the predecessor leaves
+// first.  The CUDA-core joint kernels, plain FP32, N = 2^16, n1 = 167, 32 frames, B = 1: forward
+// 30.5 ms so, 52.0 through launch_pdl.
+template <typename... Params, typename... Args>
+inline void launch_spread(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem,
+                          cudaStream_t st, Args&&... args) {
+  launch_chain(false, kernel, grid, block, smem, st, std::forward<Args>(args)...);
 }
 
 }  // namespace jtfs
