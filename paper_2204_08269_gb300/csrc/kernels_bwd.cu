@@ -580,9 +580,10 @@ k_scat1d_bwd_rows(DevPlan P, const int4* __restrict__ items, const float2* __res
   const float* g = gs2t + (((size_t)b * P.n2 + a) * P.n1 + lam0) * nt;
   const float* w = P.poolw + A.off_pw;
   float2* out = gy + (size_t)b * P.y_len + A.off_y + (size_t)(lam0 - A.lam_min) * L;
-  const int per_row = L / FB;
+  constexpr int kLogFB = FB == 8 ? 3 : (FB == 4 ? 2 : FB - 1);
+  const int logpr = logL - kLogFB, per_row = 1 << logpr;
   for (int i = threadIdx.x; i < G * per_row; i += blockDim.x) {
-    const int r = i / per_row, rest = i - r * per_row;
+    const int r = i >> logpr, rest = i & (per_row - 1);
     const int rho = rest & (tau - 1), q0 = (rest >> logtau) * FB;
     const float* gr = g + r * nt;
     // slot (j - t) mod FB holds the weight of sample j in frame t
