@@ -52,7 +52,7 @@ k_s0(DevPlan P, const float* __restrict__ x, float* __restrict__ s0) {
   float sum = 0.f, cor = 0.f;
   for (int n = part * chunk + threadIdx.x; n < (part + 1) * chunk; n += blockDim.x) {
     const int k = (int)((tT - n) & (P.N - 1));
-    const float v = xb[n], hi = __ldg(&P.phiT[k]), lo = __ldg(&P.phiT_lo[k]);
+    const float v = __ldcg(&xb[n]), hi = __ldg(&P.phiT[k]), lo = __ldg(&P.phiT_lo[k]);
     const float pr = __fmul_rn(hi, v);
     const float e = fmaf(lo, v, fmaf(hi, v, -pr));
     const float u = __fadd_rn(sum, pr);

@@ -7,16 +7,17 @@
 //  - pdl_enter, nearly all: the dependents are let go, then the predecessor's end is awaited.
 //  - pdl_enter_early: the kernel reads no result of its predecessor, only what was complete before
 //    that one let it go; it works beside the predecessor's tail and calls pdl_wait at its end.
-//    k_s0 (reads the call's input) and the contraction forms launched `late` (read Y, and G1 or the
-//    weights, as the form before them does).
+//    k_s0 (reads the call's input) and the contraction forms launched `late` (pdl_enter_form; they
+//    read Y, and G1 or the weights, as the form before them does).
 //  - pdl_enter_ordered: the wait comes before the dependents are let go.  A kernel after which an
 //    early one starts, directly or through kernels that let their dependents go at once, has to
-//    enter so: k_xfft_sub, the first kernel of every call, for k_s0 (the call's input is then
-//    complete), and the first form of a contraction stage for the later ones (Y and G1 are).
+//    enter so: k_xfft_sub, the first transform kernel of every call, for k_s0 (the call's input is
+//    then complete), and the first form of a contraction stage for the later ones (Y and G1 are).
 // griddepcontrol.wait promises visibility to the grid that executes it.  An early kernel takes over
 // what the ordered one before it was promised: the writers are complete and their results in global
-// memory when that one triggers, the early grid starts after the trigger, and the fences on
-// both sides keep its reads from any older line of an L1.  TMA reads do not go through an L1.
+// memory when that one triggers, and the early grid starts after the trigger.  Its loads must not
+// find older lines in an L1: k_s0 reads past it (__ldcg), the contraction forms through TMA (their
+// other loads are constants of the plan).
 #pragma once
 #include <cuda_runtime.h>
 
@@ -36,17 +37,14 @@ __device__ __forceinline__ void pdl_enter() {
 }
 __device__ __forceinline__ void pdl_enter_ordered() {
   pdl_wait();
-  asm volatile("fence.acq_rel.gpu;" ::: "memory");
   pdl_trigger();
 }
-__device__ __forceinline__ void pdl_enter_early() {   // pdl_wait at the kernel's end
-  asm volatile("fence.acq_rel.gpu;" ::: "memory");
-  pdl_trigger();
-}
+__device__ __forceinline__ void pdl_enter_early() { pdl_trigger(); }   // pdl_wait at its end
 // A form of a contraction stage: the first one, or a later one (late), which is independent of it,
 // starts on the SMs that it leaves and calls pdl_wait at its end.
 __device__ __forceinline__ void pdl_enter_form(int late) {
-  if (late) pdl_enter_early(); else pdl_enter_ordered();
+  if (!late) pdl_wait();
+  pdl_trigger();
 }
 
 template <typename... Params, typename... Args>
