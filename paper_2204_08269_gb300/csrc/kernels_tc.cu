@@ -872,7 +872,8 @@ k_joint_fwd_tc16(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
 // operand stages hold a whole tile's k-blocks), so the epilogue loads and frees one half while the
 // tensor cores fill the other.  With one hand-off per tile the issuer waited 839 of a tile's 2744
 // cycles for it (FP32-grade; 916 of 1717 in BF16).  B = 64, N = 2^16, FP32-grade 4.62 -> 4.44 ms;
-// BF16, B = 256, N = 2^15, 5.88 -> 5.76 ms; Eq. 4 study, B = 64, 3.35 -> 3.20 ms.  Holding the
+// BF16, B = 256, N = 2^15, 5.88 -> 5.76 ms (with roots that flushed subnormals; 6.54 with the
+// present ones); Eq. 4 study, B = 64, 3.35 -> 3.20 ms.  Holding the
 // pooling back until the next product had completed, which paid with one hand-off, cost 3 % with
 // two.  What bounds it now is the epilogue (1400 to 1550 cycles of arithmetic per tile and 500 of
 // loads, stores and waits that its sixteen warps spend in step), then the tensor pipe (about
@@ -1204,7 +1205,7 @@ k_joint_fwd_tp(const __grid_constant__ TcMaps maps, TcArgs args, DevPlan P) {
             const float2 sd = __ffma2_rn(rd, rd, __fmul2_rn(id, id));
             // roots that keep subnormal |Z|^2 (|Z| < 1.1e-19): taken as 0 they would be half the
             // instructions and quiet signals would lose their S2 (BF16, B = 256, N = 2^15: 6.62 ms
-            // so, 5.68 without; 6.31 where each row looks for such cells first, which the far
+            // so, 5.68 as 0; 6.31 where each row looks for such cells first, which the far
             // tails of short wavelets have in any signal; FP32-grade, B = 64, N = 2^16: 4.43, 4.21)
             const float2 mu = make_float2(sqrt_approx(su.x), sqrt_approx(su.y));
             const float2 md = make_float2(sqrt_approx(sd.x), sqrt_approx(sd.y));
